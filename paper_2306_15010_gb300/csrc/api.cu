@@ -73,7 +73,9 @@ ScoreWs carve_score(WsCursor &c, int H, int W, int k, int th, int tw)
     w.S = w.u16 ? (void *)c.take<uint16_t>(elems) : (void *)c.take<uint32_t>(elems);
     w.carry = c.take<int>((size_t)H * sat_strips(W) * k);
     w.bandsum = c.take<int>((size_t)sat_bands(H) * k * sat_pitch(W));
-    w.amax = c.take<unsigned long long>(1);
+    const size_t coarse = (size_t)sat_coarse_rows(H) * sat_coarse_cols(W) * sat_coarse_pitch(k);
+    w.coarse = w.u16 ? (void *)c.take<uint16_t>(coarse) : (void *)c.take<uint32_t>(coarse);
+    w.aux = c.take<ScoreAux>(1);
     return w;
 }
 
@@ -293,6 +295,17 @@ void detect_wgrid(const vqnnf_filter *bank, int F, const BankSpec &bs, WGridSpec
             // same pixels with the same weights)
             if (2 * absw >= (1ll << 31)) { memset(&ws, 0, sizeof(ws)); return; }
             ws.coef[g][q] = bs.coef[f];
+        }
+        ws.sep[g] = 1;
+        for (int q = 0; q < ws.nf[g]; ++q) {
+            const int *w = ws.w[g][q];
+            bool rows = true, cols = true;
+            for (int i = 0; i < 3; ++i) {
+                rows &= w[i] == w[3 + i] && w[i] == w[6 + i];
+                cols &= w[3 * i] == w[3 * i + 1] && w[3 * i] == w[3 * i + 2];
+            }
+            ws.rowwise[g][q] = !rows && cols;
+            ws.sep[g] &= rows || cols;
         }
     }
     ws.NG = ng;
@@ -530,16 +543,15 @@ vqnnf_status vqnnf_score(const uint8_t *q_labels, int H, int W, int k, int th, i
     memset(&wg, 0, sizeof(wg));
     if (gs.G == 0) detect_wgrid(bank, F, bs, wg);
     const bool u16 = sat_is_u16(th, tw);
-    const size_t smem = wg.NG > 0 ? score_wgrid_smem_bytes(u16 ? 2 : 4, wg, k)
-                                  : score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k);
-    if (smem > (size_t)device_smem_optin()) return VQNNF_EUNSUPPORTED;
+    if (wg.NG == 0 && score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k) > (size_t)device_smem_optin())
+        return VQNNF_EUNSUPPORTED;
     cudaStream_t s = as_stream(stream);
     WsCursor c{static_cast<char *>(ws), 0};
     ScoreWs sw = carve_score(c, H, W, k, th, tw);
-    cudaError_t e = launch_sat(q_labels, H, W, k, sw.u16, sw.carry, sw.bandsum, sw.S, s);
+    cudaError_t e = launch_sat(q_labels, H, W, k, sw.u16, sw.carry, sw.bandsum, sw.S, sw.coarse, s);
     if (e != cudaSuccess) return from_cuda(e);
     const int HO = H - th + 1, WO = W - tw + 1;
-    return from_cuda(launch_score(sw.S, sw.u16, W, k, HO, WO, bs, gs, wg, t_counts, heatmap, sw.amax,
+    return from_cuda(launch_score(sw.S, sw.coarse, sw.u16, H, W, k, HO, WO, bs, gs, wg, t_counts, heatmap, sw.aux,
                                   argmax_yx, s));
 }
 
@@ -581,9 +593,8 @@ vqnnf_status vqnnf_match_host(const float *X_host, int H, int W, int D, const fl
     memset(&wg, 0, sizeof(wg));
     if (gs.G == 0) detect_wgrid(bank, F, bs, wg);
     const bool u16 = sat_is_u16(th, tw);
-    const size_t smem = wg.NG > 0 ? score_wgrid_smem_bytes(u16 ? 2 : 4, wg, k)
-                                  : score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k);
-    if (smem > (size_t)device_smem_optin()) return VQNNF_EUNSUPPORTED;
+    if (wg.NG == 0 && score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k) > (size_t)device_smem_optin())
+        return VQNNF_EUNSUPPORTED;
     WsCursor cur{static_cast<char *>(ws), 0};
     HostWs w = carve_host(cur, H, W, D, k, th, tw, F, prec);
     const cudaStream_t s = as_stream(stream), cs = stream2 ? as_stream(stream2) : s;
@@ -618,9 +629,9 @@ vqnnf_status vqnnf_match_host(const float *X_host, int H, int W, int D, const fl
                                 nullptr, w.as, cs);
         }
         const int HO = H - th + 1, WO = W - tw + 1;
-        if (st == VQNNF_OK) st = from_cuda(launch_sat(w.ql, H, W, k, w.sc.u16, w.sc.carry, w.sc.bandsum, w.sc.S, cs));
+        if (st == VQNNF_OK) st = from_cuda(launch_sat(w.ql, H, W, k, w.sc.u16, w.sc.carry, w.sc.bandsum, w.sc.S, w.sc.coarse, cs));
         if (st == VQNNF_OK)
-            st = from_cuda(launch_score(w.sc.S, w.sc.u16, W, k, HO, WO, bs, gs, wg, w.tc, w.heat, w.sc.amax, w.am, cs));
+            st = from_cuda(launch_score(w.sc.S, w.sc.coarse, w.sc.u16, H, W, k, HO, WO, bs, gs, wg, w.tc, w.heat, w.sc.aux, w.am, cs));
         if (st == VQNNF_OK && heat_host)
             st = from_cuda(cudaMemcpyAsync(heat_host, w.heat, sizeof(float) * (size_t)HO * WO,
                                            cudaMemcpyDeviceToHost, cs));

@@ -23,9 +23,10 @@ struct FitWs {
 struct ScoreWs {
     void *S;          // integral image, uint16 (mod 2^16) or uint32, plus read slack
     bool u16;
+    void *coarse;     // its coarse samples, same type
     int *carry;
     int *bandsum;
-    unsigned long long *amax;
+    ScoreAux *aux;
 };
 
 cudaStream_t as_stream(void *s);

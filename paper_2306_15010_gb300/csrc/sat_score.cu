@@ -22,7 +22,9 @@
 //       and walks the strip's labels once per row.  Adjacent warps take adjacent strips, so
 //       the rows they write are contiguous runs.
 //
-// Score: one block per (window row, 512 windows).  The corner rows of its windows are
+// Score: score_tiles.cu goes over tiles of windows; the kernel here, for grid banks over labels too
+// incoherent for that (or images too small), visits every cluster: one block per (window row, 512
+// windows).  The corner rows of its windows are
 // staged in shared memory one cluster at a time by bulk copies (one per row segment,
 // completing on an mbarrier, four buffers in flight); each thread owns four windows and
 // accumulates exact integer L1 distances per filter over all clusters, then combines them
@@ -163,7 +165,7 @@ __device__ __forceinline__ void pack_row<uint32_t>(uint8_t *dst, const int (&acc
 template <typename T>
 __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
     const uint8_t *__restrict__ lab, int H, int W, int k, int P, int nS, int nB, const int *__restrict__ carry,
-    const int *__restrict__ bandsum, T *__restrict__ S)
+    const int *__restrict__ bandsum, T *__restrict__ S, T *__restrict__ coarse)
 {
     ptx::pdl_enter();
     constexpr int NW = SatSweep<T>::warps, PITCH = SatSweep<T>::pitch;
@@ -182,6 +184,7 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
     const int x0 = s * SW;
     const int ncolv = min(SW, P - x0);                       // S columns of the strip: a multiple of 8
     const uint32_t row_bytes = (uint32_t)(ncolv * (int)sizeof(T));   // a multiple of 16
+    const int kp = sat_coarse_pitch(k);
     const int y0 = b * BH, y1 = min(H, y0 + BH);
     const uint32_t fill = (uint32_t)(((cg + 1) * 32) & 0xFF);   // outside [32 cg, 32 cg + 31]
     const uint32_t jj = (uint32_t)j * 0x01010101u;
@@ -209,6 +212,12 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
         ptx::fence_proxy_async();
         ptx::bulk_s2g(S + ((size_t)yrow * k + j) * P + x0, st, row_bytes);
         ptx::bulk_commit();
+        if (yrow % kCoarseY == 0 || yrow == H) {              // the coarse samples of this row
+            T *c = coarse + ((size_t)((yrow + kCoarseY - 1) / kCoarseY) * sat_coarse_cols(W) + x0 / kCoarseX) * kp + j;
+#pragma unroll
+            for (int u = 0; u < SW / kCoarseX; ++u) c[(size_t)u * kp] = (T)acc[u * kCoarseX];
+            if (s == nS - 1) c[(size_t)(SW / kCoarseX) * kp] = (T)acc[SW - 1];
+        }
     };
     if (b == 0) emit(0, 1);                                   // row 0 of S (all zero)
     // labels and carry of the next row are loaded one row ahead; lane l stages columns
@@ -351,9 +360,11 @@ __global__ void __launch_bounds__(STH, G <= 3 ? 8 : 6) score_grid_kernel(const T
                                                          int HO, int WO, GridSpec gs,
                                                          const int32_t *__restrict__ tcounts,
                                                          float *__restrict__ heat,
-                                                         unsigned long long *amax)
+                                                         unsigned long long *amax, const long long *probe,
+                                                         long long dense_from)
 {
     ptx::pdl_enter();
+    if (probe && *probe <= dense_from) return;   // the tile kernel takes this image
     // For a single-rectangle filter q and clusters j, with t = template count and n = query
     // count (every pixel carries one label < k, so sum_j n_qj = area_q):
     //     L1_q = sum_j |t_qj - n_qj| = area_q + sum_{j : t_qj > 0} (|t_qj - n_qj| - n_qj)
@@ -488,224 +499,6 @@ __global__ void __launch_bounds__(STH, G <= 3 ? 8 : 6) score_grid_kernel(const T
     }
 }
 
-// Weighted-grid bank (WGridSpec): grid by grid, one pass over the clusters stages that grid's
-// four corner rows; per cluster and window the 16 corners give the 9 cell counts, each of the
-// grid's filters is their integer weighting R, and |t - R| is summed exactly per filter.  The
-// weights and coefficients are kernel parameters indexed at compile time.  After each grid's
-// pass its filters' sums enter the float heatmap accumulator (fixed order).
-template <typename T, int NG, int NCOLP>
-__global__ void __launch_bounds__(STH, 6) score_wgrid_kernel(const T *__restrict__ S, int P, int k,
-                                                          int HO, int WO, WGridSpec ws,
-                                                          const int32_t *__restrict__ tcounts,
-                                                          float *__restrict__ heat,
-                                                          unsigned long long *amax)
-{
-    ptx::pdl_enter();
-    extern __shared__ __align__(128) uint8_t smem_raw[];
-    const int ncol = ws.ncol;
-    constexpr int chunk_elems = 4 * NCOLP;                    // one cluster, four corner rows
-    T *bufs = reinterpret_cast<T *>(smem_raw);                 // [NBUF][chunk]
-    int *tc = reinterpret_cast<int *>(bufs + NBUF * chunk_elems);   // [NG][5][k]
-    uint64_t *full = reinterpret_cast<uint64_t *>(tc + NG * kMaxWFilters * k + ((NG * kMaxWFilters * k) & 1));
-    uint64_t *empty = full + NBUF;
-    int *n_issued = reinterpret_cast<int *>(empty + NBUF);
-    const int y = blockIdx.y;
-    const int x0 = blockIdx.x * TXW;
-    const int lane = threadIdx.x & 31;
-    const int nchunk = NG * k;                                 // chunk ci: grid ci / k, cluster ci % k
-    for (int q = threadIdx.x; q < NG * kMaxWFilters * k; q += blockDim.x) {
-        const int gf = q / k, j = q % k, g = gf / kMaxWFilters, f = gf % kMaxWFilters;
-        tc[q] = f < ws.nf[g] ? tcounts[(size_t)ws.filt[g][f] * k + j] : 0;
-    }
-    if (threadIdx.x == 0) {
-        for (int b = 0; b < NBUF; ++b) {
-            ptx::mbar_init(&full[b], 1);
-            ptx::mbar_init(&empty[b], STH / 32);
-        }
-        ptx::fence_barrier_init();
-        int c = 0;
-        for (; c < NBUF - 1 && c < nchunk; ++c)
-            issue_chunk<T>(bufs + c * chunk_elems, S, k, P, y, x0, c % k, ncol, NCOLP, ws.by[c / k], 4, &full[c]);
-        *n_issued = c;
-    }
-    __syncthreads();
-    float hs[WPT];
-#pragma unroll
-    for (int w = 0; w < WPT; ++w) hs[w] = 0.f;
-    bool ok = true;
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        const int nf = ws.nf[g];
-        int acc[WPT][kMaxWFilters];
-#pragma unroll
-        for (int w = 0; w < WPT; ++w)
-#pragma unroll
-            for (int f = 0; f < kMaxWFilters; ++f) acc[w][f] = 0;
-        int off[4];
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) off[cc] = ws.bx[g][cc];
-        for (int j = 0; ok && j < k; ++j) {
-            const int ch = g * k + j;
-            const int b = ch % NBUF;
-            if (threadIdx.x == 0 && ch + NBUF - 1 < nchunk) {
-                const int nb = (ch + NBUF - 1) % NBUF;
-                const int use = (ch + NBUF - 1) / NBUF;
-                if (use > 0)
-                    ok = ptx::mbar_wait_bounded(&empty[nb], (use - 1) & 1, &g_score_error, (int)VQNNF_ETIMEOUT);
-                if (ok) {
-                    const int cn = ch + NBUF - 1;
-                    issue_chunk<T>(bufs + nb * chunk_elems, S, k, P, y, x0, cn % k, ncol, NCOLP, ws.by[cn / k], 4,
-                                   &full[nb]);
-                    *n_issued = cn + 1;
-                }
-            }
-            ok = __all_sync(0xffffffffu, ok && ptx::mbar_wait_bounded(&full[b], (ch / NBUF) & 1, &g_score_error,
-                                                                      (int)VQNNF_ETIMEOUT));
-            if (!ok) break;
-            const T *cur = bufs + b * chunk_elems + threadIdx.x;
-            int t[kMaxWFilters];
-#pragma unroll
-            for (int f = 0; f < kMaxWFilters; ++f) t[f] = tc[(g * kMaxWFilters + f) * k + j];
-#pragma unroll
-            for (int w = 0; w < WPT; ++w) {
-                int cr[4][4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) cr[r][cc] = (int)cur[off[cc] + r * NCOLP + w * STH];
-                int n[9];
-#pragma unroll
-                for (int r = 0; r < 3; ++r)
-#pragma unroll
-                    for (int cc = 0; cc < 3; ++cc)
-                        n[r * 3 + cc] = box<T>(cr[r + 1][cc + 1], cr[r + 1][cc], cr[r][cc + 1], cr[r][cc]);
-#pragma unroll
-                for (int f = 0; f < kMaxWFilters; ++f) {
-                    if (f >= nf) break;
-                    int R = 0;
-#pragma unroll
-                    for (int c = 0; c < 9; ++c) R += ws.w[g][f][c] * n[c];
-                    acc[w][f] += abs(t[f] - R);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(&empty[b]))
-                                        : "memory");
-        }
-#pragma unroll
-        for (int f = 0; f < kMaxWFilters; ++f) {
-            if (f >= nf) break;
-#pragma unroll
-            for (int w = 0; w < WPT; ++w) hs[w] = fmaf(ws.coef[g][f], (float)acc[w][f], hs[w]);
-        }
-    }
-    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
-        const int issued = *n_issued;
-        for (int c = max(0, issued - NBUF); c < issued; ++c)
-            ptx::mbar_wait_bounded(&full[c % NBUF], (c / NBUF) & 1, &g_score_error, (int)VQNNF_ETIMEOUT);
-    }
-    unsigned long long best = 0ull;
-#pragma unroll
-    for (int w = 0; w < WPT; ++w) {
-        const int x = x0 + threadIdx.x + w * STH;
-        const float h = -hs[w];
-        if (ok && x < WO) {
-            heat[(size_t)y * WO + x] = h;
-            const unsigned long long key = pack_key(h, (unsigned)(y * WO + x));
-            best = key > best ? key : best;
-        }
-    }
-    if (amax) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
-        }
-        if ((threadIdx.x & 31) == 0 && best) atomicMax(amax, best);
-    }
-}
-
-// Generic bank: any weighted half-open rectangles.  Corner rows are the distinct row
-// offsets of the bank; each rectangle reads its four corners from shared memory.
-template <typename T>
-__global__ void __launch_bounds__(STH) score_generic_kernel(const T *__restrict__ S, int P, int k,
-                                                            int HO, int WO, BankSpec bs,
-                                                            const int32_t *__restrict__ tcounts,
-                                                            float *__restrict__ heat,
-                                                            unsigned long long *amax)
-{
-    ptx::pdl_enter();
-    extern __shared__ __align__(128) uint8_t smem_raw[];
-    const int ncol = bs.ncol, nrow = bs.nrow;
-    T *buf0 = reinterpret_cast<T *>(smem_raw);
-    T *buf1 = buf0 + (size_t)CH * nrow * ncol;
-    int *tc = reinterpret_cast<int *>(buf1 + (size_t)CH * nrow * ncol);      // [F][k]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(tc + bs.F * k + (bs.F * k & 1));
-    const int y = blockIdx.y;
-    const int x0 = blockIdx.x * TXW;
-    const int nchunk = (k + CH - 1) / CH;
-    for (int q = threadIdx.x; q < bs.F * k; q += blockDim.x) tc[q] = tcounts[q];
-    if (threadIdx.x == 0) {
-        ptx::mbar_init(&bar[0], 1);
-        ptx::mbar_init(&bar[1], 1);
-        ptx::fence_barrier_init();
-        issue_chunk<T>(buf0, S, k, P, y, x0, 0, ncol, ncol, bs.roff, nrow, &bar[0]);
-    }
-    __syncthreads();
-    long long l1[WPT][kMaxFilters];
-    for (int w = 0; w < WPT; ++w)
-        for (int f = 0; f < kMaxFilters; ++f) l1[w][f] = 0;
-    bool ok = true;
-    for (int ch = 0; ch < nchunk; ++ch) {
-        T *cur = (ch & 1) ? buf1 : buf0;
-        if (threadIdx.x == 0 && ch + 1 < nchunk)
-            issue_chunk<T>((ch & 1) ? buf0 : buf1, S, k, P, y, x0, (ch + 1) * CH, ncol, ncol, bs.roff, nrow,
-                           &bar[(ch + 1) & 1]);
-        ok = ptx::mbar_wait_bounded(&bar[ch & 1], (ch >> 1) & 1, &g_score_error, (int)VQNNF_ETIMEOUT);
-        if (!__syncthreads_and(ok)) { ok = false; break; }
-        const int cmax = min(CH, k - ch * CH);
-        for (int c = 0; c < cmax; ++c) {
-            const int j = ch * CH + c;
-            const T *base = cur + (size_t)c * nrow * ncol;
-            for (int f = 0; f < bs.F; ++f) {
-                const int t = tc[f * k + j];
-                for (int w = 0; w < WPT; ++w) {
-                    const int xl = threadIdx.x + w * STH;
-                    int v = 0;
-                    for (int r = bs.rect_begin[f]; r < bs.rect_begin[f + 1]; ++r) {
-                        const RectSpec rc = bs.rect[r];
-                        const T *r0 = base + rc.ry0 * ncol + xl;
-                        const T *r1 = base + rc.ry1 * ncol + xl;
-                        v += rc.weight * box<T>(r1[rc.x1], r1[rc.x0], r0[rc.x1], r0[rc.x0]);
-                    }
-                    l1[w][f] += abs(t - v);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    unsigned long long best = 0ull;
-    for (int w = 0; w < WPT; ++w) {
-        const int x = x0 + threadIdx.x + w * STH;
-        float acc = 0.f;
-        for (int f = 0; f < bs.F; ++f) acc = fmaf(bs.coef[f], (float)l1[w][f], acc);
-        const float h = -acc;
-        if (ok && x < WO) {
-            heat[(size_t)y * WO + x] = h;
-            const unsigned long long key = pack_key(h, (unsigned)(y * WO + x));
-            best = key > best ? key : best;
-        }
-    }
-    if (amax) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
-        }
-        if ((threadIdx.x & 31) == 0 && best) atomicMax(amax, best);
-    }
-}
-
 // Self-test of the bounded waits: one thread waits on an mbarrier that nothing completes.  No
 // copy is issued, so nothing is in flight when the wait gives up after `limit` SM cycles and
 // records VQNNF_ETIMEOUT in the score kernels' error word.
@@ -726,8 +519,9 @@ __global__ void argmax_finish_kernel(const unsigned long long *amax, int WO, int
 }
 
 template <typename T, int G, bool FULL>
-cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec &gs,
-                        const int32_t *tc, float *heat, unsigned long long *amax, cudaStream_t s)
+cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec &gs, const int32_t *tc,
+                        float *heat, unsigned long long *amax, const long long *probe, long long dense_from,
+                        cudaStream_t s)
 {
     BankSpec none;
     none.F = 0;
@@ -739,7 +533,7 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         {
-        const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 128>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax);
+        const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 128>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
         if (le_ != cudaSuccess) return le_;
     }
     } else {
@@ -747,7 +541,7 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         {
-        const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 256>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax);
+        const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 256>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
         if (le_ != cudaSuccess) return le_;
     }
     }
@@ -756,7 +550,7 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
 
 template <typename T>
 cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, int *bandsum, T *S,
-                         cudaStream_t s)
+                         T *coarse, cudaStream_t s)
 {
     const int nS = sat_strips(W);
     const int P = sat_pitch(W);
@@ -785,94 +579,33 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
     constexpr int NW = SatSweep<T>::warps;
     const unsigned blocks = (unsigned)((nwarps + NW - 1) / NW);
     {
-        const cudaError_t le_ = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * NW), 0, s, lab, H, W, k, P, nS, nB, carry, bandsum, S);
+        const cudaError_t le_ = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * NW), 0, s, lab, H, W, k, P, nS, nB, carry, bandsum, S, coarse);
         if (le_ != cudaSuccess) return le_;
-    }
-    return cudaGetLastError();
-}
-
-template <typename T, int NG>
-cudaError_t launch_wgrid(const T *S, int P, int k, int HO, int WO, const WGridSpec &ws, const int32_t *tc,
-                         float *heat, unsigned long long *amax, cudaStream_t s)
-{
-    const size_t smem = score_wgrid_smem_bytes(sizeof(T), ws, k);
-    dim3 grid((WO + TXW - 1) / TXW, HO);
-    cudaError_t e;
-    if (ws.ncol <= TXW + 128) {
-        e = cudaFuncSetAttribute(score_wgrid_kernel<T, NG, TXW + 128>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        {
-        const cudaError_t le_ = launch_pdl(score_wgrid_kernel<T, NG, TXW + 128>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, ws, tc, heat, amax);
-        if (le_ != cudaSuccess) return le_;
-    }
-    } else {
-        e = cudaFuncSetAttribute(score_wgrid_kernel<T, NG, TXW + 256>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        {
-        const cudaError_t le_ = launch_pdl(score_wgrid_kernel<T, NG, TXW + 256>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, ws, tc, heat, amax);
-        if (le_ != cudaSuccess) return le_;
-    }
     }
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_score_t(const T *S, int W, int k, int HO, int WO, const BankSpec &bs,
+cudaError_t launch_score_t(const T *S, const T *coarse, int H, int W, int k, int HO, int WO, const BankSpec &bs,
                            const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
-                           unsigned long long *amax, int32_t *argmax_yx, cudaStream_t s)
+                           ScoreAux *aux, cudaStream_t s)
 {
     const int P = sat_pitch(W);
+    long long dense_from = 0;
+    const ScoreRoute route = gs.G == 0 ? kScoreTiles : score_grid_route(HO, WO, k, P, gs.by[gs.G]);
     cudaError_t e = cudaSuccess;
-    if (amax) {
-        e = cudaMemsetAsync(amax, 0, sizeof(unsigned long long), s);
-        if (e != cudaSuccess) return e;
-    }
-    if ((e = record_kernel_event(VQNNF_OP_SCORE, 0, s)) != cudaSuccess) return e;
-    bool done = false;
-#define VQNNF_GRID_CASE(GG, FF)                                                         \
-    if (!done && gs.G == GG && gs.full == FF) {                                         \
-        e = launch_grid<T, GG, FF>(S, P, k, HO, WO, gs, tc, heat, amax, s);              \
-        done = true;                                                                    \
-    }
+    if (route == kScoreProbe) e = launch_score_probe(coarse, sizeof(T) == 2, W, k, HO, WO, gs, tc, aux, &dense_from, s);
+    if (e == cudaSuccess && route != kScoreDense)
+        e = launch_score_tiles(S, coarse, sizeof(T) == 2, W, k, HO, WO, bs, gs, ws, tc, heat, aux, dense_from, s);
+    if (e != cudaSuccess || route == kScoreTiles) return e;
+    const long long *probe = route == kScoreProbe ? &aux->probe : nullptr;
+#define VQNNF_GRID_CASE(GG, FF) \
+    if (gs.G == GG && gs.full == FF) return launch_grid<T, GG, FF>(S, P, k, HO, WO, gs, tc, heat, &aux->amax, probe, dense_from, s);
     VQNNF_GRID_CASE(1, false) VQNNF_GRID_CASE(1, true) VQNNF_GRID_CASE(2, false)
     VQNNF_GRID_CASE(2, true) VQNNF_GRID_CASE(3, false) VQNNF_GRID_CASE(3, true)
     VQNNF_GRID_CASE(4, false) VQNNF_GRID_CASE(4, true)
 #undef VQNNF_GRID_CASE
-    if (!done && ws.NG > 0) {
-        switch (ws.NG) {
-        case 1: e = launch_wgrid<T, 1>(S, P, k, HO, WO, ws, tc, heat, amax, s); break;
-        case 2: e = launch_wgrid<T, 2>(S, P, k, HO, WO, ws, tc, heat, amax, s); break;
-        case 3: e = launch_wgrid<T, 3>(S, P, k, HO, WO, ws, tc, heat, amax, s); break;
-        default: e = launch_wgrid<T, 4>(S, P, k, HO, WO, ws, tc, heat, amax, s); break;
-        }
-        done = true;
-    }
-    if (!done) {
-        GridSpec none;
-        none.G = 0;
-        const size_t smem = score_smem_bytes_for(sizeof(T), bs, none, k);
-        e = cudaFuncSetAttribute(score_generic_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        dim3 grid((WO + TXW - 1) / TXW, HO);
-        {
-        const cudaError_t le_ = launch_pdl(score_generic_kernel<T>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, bs, tc, heat, amax);
-        if (le_ != cudaSuccess) return le_;
-    }
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) return e;
-    if ((e = record_kernel_event(VQNNF_OP_SCORE, 1, s)) != cudaSuccess) return e;
-    if (argmax_yx && amax) {
-        {
-        const cudaError_t le_ = launch_pdl(argmax_finish_kernel, dim3(1), dim3(1), 0, s, amax, WO, argmax_yx);
-        if (le_ != cudaSuccess) return le_;
-    }
-        e = cudaGetLastError();
-    }
-    return e;
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -881,13 +614,6 @@ cudaError_t launch_score_t(const T *S, int W, int k, int HO, int WO, const BankS
 // to 256; wider templates take the generic kernel).
 int score_grid_pitch(int ncol) { return ncol <= TXW + 128 ? TXW + 128 : TXW + 256; }
 bool score_grid_fits(int ncol) { return ncol <= TXW + 256; }
-
-size_t score_wgrid_smem_bytes(size_t elem, const WGridSpec &ws, int k)
-{
-    return elem * (size_t)NBUF * 4 * score_grid_pitch(ws.ncol) + sizeof(int) * ((size_t)ws.NG * kMaxWFilters * k + 1) +
-           sizeof(uint64_t) * 2 * NBUF + 16 + 16;
-}
-
 
 size_t score_smem_bytes_for(size_t elem, const BankSpec &bs, const GridSpec &gs, int k)
 {
@@ -908,10 +634,12 @@ int score_ncol(int tw) { return (TXW + tw + 7) / 8 * 8; }
 size_t sat_slack_elems(int tw) { return (size_t)score_ncol(tw) + 64; }
 
 cudaError_t launch_sat(const uint8_t *lab, int H, int W, int k, bool u16, int *carry, int *bandsum,
-                       void *S, cudaStream_t s)
+                       void *S, void *coarse, cudaStream_t s)
 {
-    return u16 ? launch_sat_t<uint16_t>(lab, H, W, k, carry, bandsum, static_cast<uint16_t *>(S), s)
-               : launch_sat_t<uint32_t>(lab, H, W, k, carry, bandsum, static_cast<uint32_t *>(S), s);
+    return u16 ? launch_sat_t<uint16_t>(lab, H, W, k, carry, bandsum, static_cast<uint16_t *>(S),
+                                        static_cast<uint16_t *>(coarse), s)
+               : launch_sat_t<uint32_t>(lab, H, W, k, carry, bandsum, static_cast<uint32_t *>(S),
+                                        static_cast<uint32_t *>(coarse), s);
 }
 
 cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, const BankSpec &bs,
@@ -925,14 +653,21 @@ cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_score(const void *S, bool u16, int W, int k, int HO, int WO, const BankSpec &bs,
-                         const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
-                         unsigned long long *amax, int32_t *argmax_yx, cudaStream_t s)
+cudaError_t launch_score(const void *S, const void *coarse, bool u16, int H, int W, int k, int HO, int WO,
+                         const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
+                         ScoreAux *aux, int32_t *argmax_yx, cudaStream_t s)
 {
-    return u16 ? launch_score_t<uint16_t>(static_cast<const uint16_t *>(S), W, k, HO, WO, bs, gs, ws, tc,
-                                          heat, amax, argmax_yx, s)
-               : launch_score_t<uint32_t>(static_cast<const uint32_t *>(S), W, k, HO, WO, bs, gs, ws, tc,
-                                          heat, amax, argmax_yx, s);
+    cudaError_t e = cudaMemsetAsync(aux, 0, 16, s);                    // the maximum and the probe
+    if (e != cudaSuccess) return e;
+    if ((e = record_kernel_event(VQNNF_OP_SCORE, 0, s)) != cudaSuccess) return e;
+    e = u16 ? launch_score_t(static_cast<const uint16_t *>(S), static_cast<const uint16_t *>(coarse), H, W, k, HO, WO, bs,
+                             gs, ws, tc, heat, aux, s)
+            : launch_score_t(static_cast<const uint32_t *>(S), static_cast<const uint32_t *>(coarse), H, W, k, HO, WO, bs,
+                             gs, ws, tc, heat, aux, s);
+    if (e != cudaSuccess) return e;
+    if ((e = record_kernel_event(VQNNF_OP_SCORE, 1, s)) != cudaSuccess) return e;
+    if (argmax_yx) e = launch_pdl(argmax_finish_kernel, dim3(1), dim3(1), 0, s, &aux->amax, WO, argmax_yx);
+    return e;
 }
 
 cudaError_t launch_wait_selftest(long long limit_cycles, cudaStream_t s)

@@ -59,10 +59,19 @@ struct WGridSpec {
     int w[kMaxWGrids][kMaxWFilters][9];       // cell weights, cell r * 3 + c
     int filt[kMaxWGrids][kMaxWFilters];       // bank index of the filter
     float coef[kMaxWGrids][kMaxWFilters];     // w_f / A_f
+    int sep[kMaxWGrids];                      // every filter of the grid has equal rows or equal columns
+    int rowwise[kMaxWGrids][kMaxWFilters];    // sep: 1 = weights by row w[3 r], 0 = weights by column w[c]
 };
 
 size_t score_smem_bytes_for(size_t elem, const BankSpec &bs, const GridSpec &gs, int k);
-size_t score_wgrid_smem_bytes(size_t elem, const WGridSpec &ws, int k);
+// Coarse samples of the integral image, cluster by cluster: S at rows 0, 8, 16, .. and H and at
+// columns 0, 16, 32, .. and the last, element ((row index) * columns + column index) * kp + j,
+// kp = k rounded up to a multiple of 4.  One coalesced read per corner tells for many clusters
+// whether a region rounded out to the samples holds them.
+constexpr int kCoarseX = 16, kCoarseY = 8;
+__host__ __device__ inline int sat_coarse_cols(int W) { return (W + 64) / 64 * (64 / kCoarseX) + 1; }
+__host__ __device__ inline int sat_coarse_pitch(int k) { return (k + 3) / 4 * 4; }
+__host__ __device__ inline int sat_coarse_rows(int H) { return (H + kCoarseY - 1) / kCoarseY + 1; }
 bool sat_is_u16(int th, int tw);
 int sat_pitch(int W);
 int sat_strips(int W);
@@ -71,12 +80,31 @@ int score_ncol(int tw);
 bool score_grid_fits(int ncol);   // the grid kernel stages at most TXW + 256 columns
 size_t sat_slack_elems(int tw);
 cudaError_t launch_sat(const uint8_t *lab, int H, int W, int k, bool u16, int *carry, int *bandsum,
-                       void *S, cudaStream_t s);
+                       void *S, void *coarse, cudaStream_t s);
 cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, const BankSpec &bs,
                                     int32_t *counts, cudaStream_t s);
-cudaError_t launch_score(const void *S, bool u16, int W, int k, int HO, int WO, const BankSpec &bs,
-                         const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
-                         unsigned long long *amax, int32_t *argmax_yx, cudaStream_t s);
+// Device words of one score: the maximum's key and the probe (both start at zero), and the grid
+// bank's template side.
+constexpr int kMaxSlots = 17;
+struct ScoreAux {
+    unsigned long long amax;
+    long long probe;                              // > dense_from: the dense kernel is cheaper
+    int tsum[kMaxSlots];                          // per slot: sum of the positive template counts
+    alignas(16) int t[kMaxSlots][256];            // the slots' template counts
+};
+cudaError_t launch_score(const void *S, const void *coarse, bool u16, int H, int W, int k, int HO, int WO,
+                         const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
+                         ScoreAux *aux, int32_t *argmax_yx, cudaStream_t s);
+// Which kernel scores a grid bank: the dense kernel, or the one that a probe of the image's tiles
+// finds cheaper (score_tiles.cu); any other bank goes over tiles.
+enum ScoreRoute { kScoreTiles, kScoreDense, kScoreProbe };
+ScoreRoute score_grid_route(int HO, int WO, int k, int P, int th);
+cudaError_t launch_score_probe(const void *coarse, bool u16, int W, int k, int HO, int WO, const GridSpec &gs,
+                               const int32_t *tc, ScoreAux *aux, long long *dense_from, cudaStream_t s);
+// A grid bank only where aux->probe <= dense_from, after the probe.
+cudaError_t launch_score_tiles(const void *S, const void *coarse, bool u16, int W, int k, int HO, int WO,
+                               const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
+                               ScoreAux *aux, long long dense_from, cudaStream_t s);
 cudaError_t read_and_clear_score_error(int *out);
 // One-thread kernel whose mbarrier wait gives up after limit_cycles (self-test of the bounded
 // waits; sets the error word that read_and_clear_score_error returns).

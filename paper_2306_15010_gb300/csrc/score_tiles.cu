@@ -1,0 +1,743 @@
+// Eq. 2 score over tiles of windows, visiting only the clusters that both images hold there.
+//
+// A warp owns a tile of 32 NX x TY windows.  For a rectangle of the bank and a cluster j, let t be
+// the template's count and n the count of a window of the query.  Then
+//     sum_j |t_j - n_j| = area + sum_{t_j > 0} t_j - 2 sum_{t_j > 0} min(t_j, n_j)
+// (every query pixel carries one label, so sum_j n_j = area), and min(t_j, n_j) = 0 for every
+// window of the tile when the rectangle, swept over the tile, meets no pixel labelled j.  A
+// four-corner sum of the integral image over the swept region, rounded out to the coarse samples,
+// tells; a sum of zero is proof, so skipping is exact.  Labels are piecewise constant: on the
+// 2048 x 2048, k = 128 workload with a 128 x 128 template about 95 of the 1,280 (rectangle,
+// cluster) pairs of a 64 x 4 tile remain, against 486 that the template's counts alone leave.  The
+// other two bank forms use the same test with the box of a grid or a filter: a cluster that is
+// absent adds |t|.
+//
+// What bounds it: instruction issue and the corner rows' way from L2 into shared memory, in that
+// order (ncu, 2048 x 2048: 70 % and 60 % of peak before the pair list, 2.3 KB per pair and tile).
+// Tiles of 64 x 4 windows with three staged pairs and 14 blocks per SM take 0.45 ms there; 64 x 8
+// took 0.46 to 0.51, 128 x 4 0.52, 32 x 4 0.54 ms, two staged pairs 0.49 ms, loads from global memory
+// straight into registers 0.48 ms and more, a table laid out by 64-column strips the same.  The
+// dense kernel (sat_score.cu: every cluster, staged for 512 windows) takes 1.13 ms.  Testing against
+// the full-size table (a gather from 32 planes per corner) cost 0.34 ms by itself, against the
+// coarse samples 0.06 ms; they leave 101 pairs where the exact region leaves 93.
+#include "common.cuh"
+#include "ptx.cuh"
+#include "score_spec.cuh"
+
+namespace vqnnf {
+namespace {
+
+constexpr int TW = 2;              // warps per block, their tiles side by side in x
+constexpr int NST = 3;             // staged pairs of a warp
+
+__device__ __forceinline__ unsigned long long pack_key(float v, unsigned idx)
+{
+    unsigned b = __float_as_uint(v);
+    b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // order-preserving
+    return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - idx);
+}
+
+// Box count from four integral-image values; exact mod 2^16 for the 16-bit table.
+template <typename T>
+__device__ __forceinline__ int box(int s11, int s10, int s01, int s00)
+{
+    const int v = s11 - s10 - s01 + s00;
+    return sizeof(T) == 2 ? (v & 0xFFFF) : v;
+}
+
+// The integral image, element (y, j, x) at (y * k + j) * P + x, and its coarse samples.
+template <typename T>
+struct Sat {
+    const T *S, *coarse;
+    int P, k, ccols, kp;
+};
+
+// The clusters that the region [x0, x1) x [y0, y1) of the image, rounded out to the coarse
+// samples, holds.
+template <typename T>
+struct Region {
+    const T *p00, *p01, *p10, *p11;
+    __device__ __forceinline__ Region(const Sat<T> &s, int x0, int y0, int x1, int y1)
+    {
+        const int cx0 = x0 / kCoarseX, cx1 = (x1 + kCoarseX - 1) / kCoarseX;
+        const T *top = s.coarse + (size_t)(y0 / kCoarseY) * s.ccols * s.kp;
+        const T *bot = s.coarse + (size_t)((y1 + kCoarseY - 1) / kCoarseY) * s.ccols * s.kp;
+        p00 = top + (size_t)cx0 * s.kp, p01 = top + (size_t)cx1 * s.kp;
+        p10 = bot + (size_t)cx0 * s.kp, p11 = bot + (size_t)cx1 * s.kp;
+    }
+    // bit u: cluster j + u, j a multiple of 4
+    __device__ __forceinline__ unsigned holds4(int j) const
+    {
+        struct __align__(4 * sizeof(T)) Four { T v[4]; };
+        const Four a = *reinterpret_cast<const Four *>(p11 + j), b = *reinterpret_cast<const Four *>(p10 + j);
+        const Four c = *reinterpret_cast<const Four *>(p01 + j), d = *reinterpret_cast<const Four *>(p00 + j);
+        unsigned h = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h |= (box<T>(a.v[u], b.v[u], c.v[u], d.v[u]) != 0 ? 1u : 0u) << u;
+        return h;
+    }
+};
+
+// Whether the count of a region of w x h pixels, rounded out, stays below the table's modulus (one
+// that could reach it is not tested: every cluster is visited).
+template <typename T>
+__host__ __device__ inline bool testable(int w, int h)
+{
+    return sizeof(T) > 2 || (long long)(w + 2 * (kCoarseX - 1)) * (h + 2 * (kCoarseY - 1)) <= 65535;
+}
+
+// The clusters a tile visits, as bits: word g = 4 G + u, bit b is cluster 128 G + 4 b + u (a lane
+// reads four clusters' samples at once).  Here: those that the region holds, or every one where
+// the region is not tested.
+template <typename T>
+__device__ __forceinline__ void visit_words(unsigned *act, int k, bool test, const Region<T> &reg)
+{
+    const int lane = threadIdx.x & 31;
+    for (int j0 = 0; j0 < k; j0 += 128) {
+        const int j = j0 + 4 * lane;
+        const unsigned h = j >= k ? 0u : test ? reg.holds4(j) : 15u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned m = __ballot_sync(0xffffffffu, j + u < k && ((h >> u) & 1u));
+            if (lane == 0) act[j0 / 32 + u] = m;
+        }
+    }
+}
+__device__ __forceinline__ int word_cluster(int w, unsigned m) { return 128 * (w >> 2) + 4 * (__ffs(m) - 1) + (w & 3); }
+__device__ __forceinline__ int words_of(int k) { return (k + 127) / 128 * 4; }
+
+// Corner rows and columns of a grid bank's slot: cell q, or the full window (q = G G).
+struct Slot {
+    int x0, x1, y0, y1;
+    __device__ __forceinline__ Slot(const GridSpec &gs, int q)
+    {
+        const int G = gs.G;
+        const bool full = q == G * G;
+        x0 = gs.bx[full ? 0 : q % G], x1 = gs.bx[full ? G : q % G + 1];
+        y0 = gs.by[full ? 0 : q / G], y1 = gs.by[full ? G : q / G + 1];
+    }
+};
+
+__device__ __forceinline__ void warp_argmax(unsigned long long best, unsigned long long *amax)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+        best = other > best ? other : best;
+    }
+    if ((threadIdx.x & 31) == 0 && best) atomicMax(amax, best);
+}
+
+// Writes this lane's column of the tile; the larger of `best` and its values' keys.
+template <int TY>
+__device__ __forceinline__ unsigned long long put_tile(const float (&hs)[TY], int X, int Y0, int WO,
+                                                       float *__restrict__ heat, unsigned long long best)
+{
+    if (X < WO) {
+#pragma unroll
+        for (int r = 0; r < TY; ++r) {
+            const unsigned idx = (unsigned)((Y0 + r) * WO + X);
+            heat[idx] = -hs[r];
+            const unsigned long long key = pack_key(-hs[r], idx);
+            best = key > best ? key : best;
+        }
+    }
+    return best;
+}
+
+// Asynchronous copies of 16 (past L1) and 4 bytes into shared memory, in commit groups.
+__device__ __forceinline__ void cp16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp4(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Grid bank: the shape of a warp's tile and of one staged pair: the four corner blocks of TY rows,
+// each row 32 NX columns from a 16-byte boundary on.
+template <typename T, int NX, int TY>
+struct GridTile {
+    static constexpr int E = 16 / (int)sizeof(T);            // elements of a 16-byte chunk
+    static constexpr int CPR = 32 * NX / E + 1;              // chunks per row
+    static constexpr int NCH = 4 * TY * CPR;                 // chunks per pair
+    static constexpr int PER = (NCH + 31) / 32;              // per lane
+    static constexpr int STAGE = NCH * 16;
+};
+// A pair to visit: slot, cluster and template count (below 2^16 where the table is 16-bit: a
+// template of at most 65,535 pixels).
+template <typename T> struct PairOf;
+template <> struct PairOf<uint16_t> {
+    uint32_t v;
+    PairOf() = default;
+    __device__ __forceinline__ PairOf(int q, int j, int t) : v((uint32_t)t << 16 | (uint32_t)q << 8 | (uint32_t)j) {}
+    __device__ __forceinline__ int t() const { return (int)(v >> 16); }
+    __device__ __forceinline__ int q() const { return (int)(v >> 8 & 255u); }
+    __device__ __forceinline__ int j() const { return (int)(v & 255u); }
+};
+template <> struct PairOf<uint32_t> {
+    uint2 v;
+    PairOf() = default;
+    __device__ __forceinline__ PairOf(int q, int j, int t) : v(make_uint2((uint32_t)q << 8 | (uint32_t)j, (uint32_t)t)) {}
+    __device__ __forceinline__ int t() const { return (int)v.y; }
+    __device__ __forceinline__ int q() const { return (int)(v.x >> 8); }
+    __device__ __forceinline__ int j() const { return (int)(v.x & 255u); }
+};
+constexpr int kGridY = 4;         // window rows of a grid bank's tile, 64 wide
+constexpr int kPairs = 512;        // a warp's list: at least the pairs of four slots of 128 clusters
+
+// `test`: the slots whose region is tested.
+template <typename T, int NX, int TY>
+__global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 14 : 1) score_grid_tile_kernel(Sat<T> sat, int HO, int WO, GridSpec gs, unsigned test,
+                                                                  float *__restrict__ heat, ScoreAux *aux,
+                                                                  long long dense_from)
+{
+    using L = GridTile<T, NX, TY>;
+    ptx::pdl_enter();
+    if (aux->probe > dense_from) return;                     // the dense kernel takes this image
+    __shared__ __align__(16) uint8_t stage_s[TW][NST][L::STAGE];
+    __shared__ PairOf<T> list_s[TW][kPairs];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int nslot = gs.G * gs.G + gs.full, k = sat.k;
+    const int X0 = ((int)blockIdx.x * TW + wi) * 32 * NX;
+    if (X0 >= WO) return;                                    // uniform over the warp
+    const int Y0 = min((int)blockIdx.y * TY, HO - TY);       // the last tile moves up to stay whole
+    const int xe = min(X0 + 32 * NX - 1, WO - 1);            // last window column of the tile
+    PairOf<T> *list = list_s[wi];
+    // the tile's rows start here; offsets from it in 16-byte units stay below 2^32 (checked on the host)
+    const uint4 *S16 = reinterpret_cast<const uint4 *>(sat.S + (size_t)Y0 * k * sat.P);
+    const uint32_t plane16 = (uint32_t)(sat.P / L::E);
+    uint32_t off[L::PER];                                    // this lane's chunks of a slot
+    float hs[NX][TY];
+    int acc[NX][TY];
+#pragma unroll
+    for (int c = 0; c < NX; ++c)
+#pragma unroll
+        for (int r = 0; r < TY; ++r) hs[c][r] = 0.f, acc[c][r] = 0;
+    auto fold = [&](int q) {                                  // H = - sum_q coef_q L1_q, slot by slot
+        const float coef = gs.slot_coef[q];
+        const int base = gs.slot_area[q] + aux->tsum[q];
+#pragma unroll
+        for (int c = 0; c < NX; ++c)
+#pragma unroll
+            for (int r = 0; r < TY; ++r) {
+                hs[c][r] = fmaf(coef, (float)(base - 2 * acc[c][r]), hs[c][r]);
+                acc[c][r] = 0;
+            }
+    };
+    const uint32_t st0 = ptx::smem_u32(stage_s[wi][0]) + lane * 16;
+    const T *sm = reinterpret_cast<const T *>(stage_s[wi][0]) + lane;
+    int q = 0, da = 0, db = 0;                               // slot; its columns' places in their staged rows
+    bool entered = false;
+    auto visit = [&](int n) {
+        int iq = -1, ib = 0;
+        auto issue = [&](int p) {
+            if (p < n) {
+                const PairOf<T> e = list[p];
+                if (e.q() != iq) {
+                    iq = e.q();
+                    const Slot sl(gs, iq);
+                    const int xa = (X0 + sl.x0) & ~(L::E - 1), xb = (X0 + sl.x1) & ~(L::E - 1);
+#pragma unroll
+                    for (int i = 0; i < L::PER; ++i) {
+                        const int idx = lane + 32 * i, row = idx / L::CPR, ch = idx % L::CPR;
+                        const int blk = row / TY, r = row % TY;   // blocks: top a, top b, bottom a, bottom b
+                        const int x = min(((blk & 1) ? xb : xa) + ch * L::E, sat.P - L::E);
+                        const int y = ((blk & 2) ? sl.y1 : sl.y0) + r;
+                        off[i] = (uint32_t)y * (uint32_t)k * plane16 + (uint32_t)(x / L::E);
+                    }
+                }
+                const uint4 *src = S16 + (uint32_t)e.j() * plane16;
+                const uint32_t dst = st0 + (uint32_t)ib * L::STAGE;
+#pragma unroll
+                for (int i = 0; i < L::PER; ++i)
+                    if (32 * i + 32 <= L::NCH || lane + 32 * i < L::NCH) cp16(dst + 32 * 16 * i, src + off[i]);
+            }
+            cp_commit();
+            ib = ib + 1 < NST ? ib + 1 : 0;
+        };
+#pragma unroll
+        for (int p = 0; p < NST - 1; ++p) issue(p);
+        int b = 0;
+        for (int p = 0; p < n; ++p) {
+            cp_wait<NST - 2>();
+            __syncwarp();                                    // every lane's copies have landed, the oldest buffer is read
+            issue(p + NST - 1);
+            const PairOf<T> e = list[p];
+            if (e.q() != q || !entered) {
+                while (q < e.q()) fold(q++);
+                entered = true;
+                const Slot sl(gs, q);
+                da = (X0 + sl.x0) & (L::E - 1);
+                db = (X0 + sl.x1) & (L::E - 1);
+            }
+            const int t = e.t();
+            constexpr int RP = L::CPR * L::E;                // elements between rows
+            const T *ta = sm + b * (L::STAGE / (int)sizeof(T)) + da, *tb = sm + b * (L::STAGE / (int)sizeof(T)) + db;
+#pragma unroll
+            for (int c = 0; c < NX; ++c)
+#pragma unroll
+                for (int r = 0; r < TY; ++r)
+                    acc[c][r] += min(t, box<T>(tb[(3 * TY + r) * RP + 32 * c], ta[(2 * TY + r) * RP + 32 * c],
+                                               tb[(TY + r) * RP + 32 * c], ta[r * RP + 32 * c]));
+            b = b + 1 < NST ? b + 1 : 0;
+        }
+        __syncwarp();                                        // the list may be rewritten
+    };
+    // the clusters to visit, four words' samples in flight at a time: four slots of at most 128
+    // clusters, or two of more
+    constexpr int QB = 4;
+    const int two = k > 128, qb = QB >> two;
+    int n = 0;
+    for (int q0 = 0; q0 < nslot; q0 += qb) {
+        unsigned h[QB];
+        int4 t[QB];
+#pragma unroll
+        for (int i = 0; i < QB; ++i) {
+            const int s = min(q0 + (i >> two), nslot - 1), j = 128 * (i & two) + 4 * lane;
+            const Slot sl(gs, s);
+            const Region<T> reg(sat, X0 + sl.x0, Y0 + sl.y0, xe + sl.x1, Y0 + TY - 1 + sl.y1);
+            h[i] = j >= k || q0 + (i >> two) >= nslot ? 0u : (test >> s) & 1 ? reg.holds4(j) : 15u;
+            t[i] = *reinterpret_cast<const int4 *>(&aux->t[s][j]);
+        }
+        int cnt = 0;
+#pragma unroll
+        for (int i = 0; i < QB; ++i) {
+            h[i] &= (t[i].x > 0 ? 1u : 0u) | (t[i].y > 0 ? 2u : 0u) | (t[i].z > 0 ? 4u : 0u) | (t[i].w > 0 ? 8u : 0u);
+            cnt += __popc(h[i]);
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (n + cnt > kPairs) {
+            __syncwarp();
+            visit(n);
+            n = 0;
+        }
+#pragma unroll
+        for (int i = 0; i < QB; ++i) {
+            const int s = q0 + (i >> two), j = 128 * (i & two) + 4 * lane;
+            const int tv[4] = {t[i].x, t[i].y, t[i].z, t[i].w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned m = __ballot_sync(0xffffffffu, (h[i] >> u) & 1u);
+                if ((h[i] >> u) & 1u) list[n + __popc(m & ((1u << lane) - 1u))] = PairOf<T>(s, j + u, tv[u]);
+                n += __popc(m);
+            }
+        }
+    }
+    __syncwarp();
+    visit(n);
+    while (q < nslot) fold(q++);
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int c = 0; c < NX; ++c) best = put_tile<TY>(hs[c], X0 + 32 * c + lane, Y0, WO, heat, best);
+    warp_argmax(best, &aux->amax);
+}
+
+// Weighted-grid bank (WGridSpec): grid by grid, the clusters present in the grid's box add
+// |t - R| - |t| to a filter's sum_j |t_j|, R the filter's integer weighting of the cell counts.
+// Where every filter weights whole columns or whole rows of cells (the Gaussian and Haar filters
+// with equal bin weights: SEP), the three column and three row counts come from the 12 corners on
+// the box's edge; otherwise the nine cell counts from all 16.  A staged (grid, cluster) is the four
+// boundary rows' TY rows, each from the first boundary column on; two lanes copy a row.
+// On a 720 x 1280 query (k = 128, the paper's 15 filters, 97 x 82 template) 0.28 ms, against 2.25 ms
+// for the kernel that visited every cluster and took all nine cells; with three stages 0.33 ms, with
+// tiles of 64 x 4 windows and the grids unrolled 0.67 ms (fewer warps, instruction cache).  It stays
+// the faster one on labels without any coherence (1.44 against 2.26 ms).
+constexpr int kWX = 1, kWY = 4;    // tile: 32 kWX x kWY windows
+#ifndef WNSTV
+#define WNSTV 2
+#endif
+constexpr int WNST = WNSTV;
+template <typename T>
+struct WTile {
+    static constexpr int E = 16 / (int)sizeof(T);
+    // 16-byte chunks of a staged row for a grid `w` columns wide (any alignment), an even number
+    static int chunks(int w) { return ((w + 32 * kWX + E - 1 + E - 1) / E + 1) / 2 * 2; }
+    // shared-memory bytes of one stage: the rows and the template counts
+    static size_t stage(int ch) { return (size_t)16 * 4 * kWY * ch + 32; }
+};
+
+template <typename T, bool SEP>
+__global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, int HO, int WO, WGridSpec ws, unsigned test,
+                                                                   int nch, const int32_t *__restrict__ tcounts,
+                                                                   float *__restrict__ heat, unsigned long long *amax)
+{
+    constexpr int E = WTile<T>::E, NX = kWX, TY = kWY;
+    static_assert(TY == 4, "two lanes copy each of the 4 x TY staged rows");
+    ptx::pdl_enter();
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint16_t list_s[TW][kMaxWGrids * kMaxK];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int k = sat.k, NG = ws.NG;
+    const int X0 = ((int)blockIdx.x * TW + wi) * 32 * NX;
+    if (X0 >= WO) return;
+    const int Y0 = min((int)blockIdx.y * TY, HO - TY);
+    const int xe = min(X0 + 32 * NX - 1, WO - 1);
+    uint16_t *list = list_s[wi];                             // grid << 8 | cluster, grid by grid
+    int n = 0;
+    for (int g = 0; g < NG; ++g) {
+        const Region<T> reg(sat, X0 + ws.bx[g][0], Y0 + ws.by[g][0], xe + ws.bx[g][3], Y0 + TY - 1 + ws.by[g][3]);
+        for (int j0 = 0; j0 < k; j0 += 128) {
+            const int j = j0 + 4 * lane;
+            const unsigned h = j >= k ? 0u : (test >> g) & 1 ? reg.holds4(j) : 15u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool v = j + u < k && ((h >> u) & 1u);
+                const unsigned m = __ballot_sync(0xffffffffu, v);
+                if (v) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(g << 8 | (j + u));
+                n += __popc(m);
+            }
+        }
+    }
+    __syncwarp();
+    const uint32_t stage = 16 * 4 * TY * nch + 32;
+    uint8_t *mine = smem + (size_t)wi * WNST * stage;
+    const uint32_t st0 = ptx::smem_u32(mine);
+    int ig = -1, nc = 0, ib = 0;                             // grid of the copies, its chunks per row
+    const T *row = nullptr;
+    auto issue = [&](int p) {
+        if (p < n) {
+            const int g = list[p] >> 8, j = list[p] & 255;
+            if (g != ig) {
+                ig = g;
+                const int xa = (X0 + ws.bx[g][0]) & ~(E - 1);
+                // chunks up to the last corner column; none starts past the table's row
+                nc = (min(X0 + 32 * NX - 1 + ws.bx[g][3], sat.P - 1) - xa) / E + 1;
+                row = sat.S + (size_t)(Y0 + ws.by[g][lane >> 3] + ((lane >> 1) & 3)) * k * sat.P + xa + (lane & 1) * E;
+            }
+            const uint32_t st = st0 + (uint32_t)ib * stage;
+            uint32_t dst = st + (uint32_t)((lane >> 1) * nch + (lane & 1)) * 16;
+            const T *src = row + (size_t)j * sat.P;
+            for (int c = lane & 1; c < nc; c += 2, dst += 32, src += 2 * E) cp16(dst, src);
+            if (lane < ws.nf[g]) cp4(st + 16 * 4 * TY * nch + 4 * lane, tcounts + (size_t)ws.filt[g][lane] * k + j);
+        }
+        cp_commit();
+        ib = ib + 1 < WNST ? ib + 1 : 0;
+    };
+    float hs[NX][TY];
+#pragma unroll
+    for (int c = 0; c < NX; ++c)
+#pragma unroll
+        for (int r = 0; r < TY; ++r) hs[c][r] = 0.f;
+#pragma unroll
+    for (int p = 0; p < WNST - 1; ++p) issue(p);
+    int p = 0, b = 0;
+    const int rp = nch * E, d = TY * rp;                     // elements to the next staged row, to the next boundary row
+#pragma unroll 1
+    for (int g = 0; g < NG; ++g) {
+        const int nf = ws.nf[g];
+        int acc[kMaxWFilters][NX][TY];
+#pragma unroll
+        for (int f = 0; f < kMaxWFilters; ++f) {
+            int ts = 0;
+            if (f < nf) {
+                const int32_t *tc = tcounts + (size_t)ws.filt[g][f] * k;
+                for (int j = lane; j < k; j += 32) ts += abs(tc[j]);
+                ts = __reduce_add_sync(0xffffffffu, ts);
+            }
+#pragma unroll
+            for (int c = 0; c < NX; ++c)
+#pragma unroll
+                for (int r = 0; r < TY; ++r) acc[f][c][r] = ts;
+        }
+        int col[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) col[c] = lane + ws.bx[g][c] - ws.bx[g][0] + ((X0 + ws.bx[g][0]) & (E - 1));
+#pragma unroll 1
+        for (; p < n && (list[p] >> 8) == g; ++p) {
+            cp_wait<WNST - 2>();
+            __syncwarp();
+            issue(p + WNST - 1);
+            const T *v = reinterpret_cast<const T *>(mine + (size_t)b * stage);
+            const int *ts = reinterpret_cast<const int *>(mine + (size_t)b * stage + 16 * 4 * TY * nch);
+            constexpr int NN = SEP ? 6 : 9;
+            int m[NX][TY][NN];                               // column and row counts, or cell counts
+#pragma unroll
+            for (int r = 0; r < TY; ++r)
+#pragma unroll
+                for (int c = 0; c < NX; ++c) {
+                    const T *e = v + r * rp + 32 * c;
+                    if (SEP) {
+                        int top[4], bot[4], lft[4], rgt[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            top[i] = (int)e[col[i]];
+                            bot[i] = (int)e[3 * d + col[i]];
+                        }
+                        lft[0] = top[0], rgt[0] = top[3], lft[3] = bot[0], rgt[3] = bot[3];
+#pragma unroll
+                        for (int i = 1; i < 3; ++i) {
+                            lft[i] = (int)e[i * d + col[0]];
+                            rgt[i] = (int)e[i * d + col[3]];
+                        }
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            m[c][r][i] = box<T>(bot[i + 1], bot[i], top[i + 1], top[i]);
+                            m[c][r][3 + i] = box<T>(rgt[i + 1], lft[i + 1], rgt[i], lft[i]);
+                        }
+                    } else {
+                        int cr[4][4];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) cr[a][i] = (int)e[a * d + col[i]];
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+#pragma unroll
+                            for (int i = 0; i < 3; ++i)
+                                m[c][r][(a * 3 + i) % NN] = box<T>(cr[a + 1][i + 1], cr[a + 1][i], cr[a][i + 1], cr[a][i]);
+                    }
+                }
+#pragma unroll
+            for (int f = 0; f < kMaxWFilters; ++f) {
+                if (f >= nf) break;
+                const int t = ts[f], at = abs(t);
+                if (SEP && ws.rowwise[g][f]) {
+                    const int w0 = ws.w[g][f][0], w1 = ws.w[g][f][3], w2 = ws.w[g][f][6];
+#pragma unroll
+                    for (int c = 0; c < NX; ++c)
+#pragma unroll
+                        for (int r = 0; r < TY; ++r)
+                            acc[f][c][r] += abs(t - (w0 * m[c][r][3] + w1 * m[c][r][4] + w2 * m[c][r][5])) - at;
+                } else if (SEP) {
+                    const int w0 = ws.w[g][f][0], w1 = ws.w[g][f][1], w2 = ws.w[g][f][2];
+#pragma unroll
+                    for (int c = 0; c < NX; ++c)
+#pragma unroll
+                        for (int r = 0; r < TY; ++r)
+                            acc[f][c][r] += abs(t - (w0 * m[c][r][0] + w1 * m[c][r][1] + w2 * m[c][r][2])) - at;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < NX; ++c)
+#pragma unroll
+                        for (int r = 0; r < TY; ++r) {
+                            int R = 0;
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) R += ws.w[g][f][i] * m[c][r][i % NN];
+                            acc[f][c][r] += abs(t - R) - at;
+                        }
+                }
+            }
+            b = b + 1 < WNST ? b + 1 : 0;
+        }
+#pragma unroll
+        for (int f = 0; f < kMaxWFilters; ++f) {
+            if (f >= nf) break;
+#pragma unroll
+            for (int c = 0; c < NX; ++c)
+#pragma unroll
+                for (int r = 0; r < TY; ++r) hs[c][r] = fmaf(ws.coef[g][f], (float)acc[f][c][r], hs[c][r]);
+        }
+    }
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int c = 0; c < NX; ++c) best = put_tile<TY>(hs[c], X0 + 32 * c + lane, Y0, WO, heat, best);
+    warp_argmax(best, amax);
+}
+
+// Any bank (weighted half-open rectangles, filter by filter), and the weighted grids of images with
+// fewer than kWY window rows: corners straight from global memory.  Sums in 64 bits: only each
+// filter's counts are known to fit 32.
+template <typename T, int TY>
+__global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int HO, int WO, BankSpec bs,
+                                                                const int32_t *__restrict__ tcounts,
+                                                                float *__restrict__ heat, unsigned long long *amax)
+{
+    ptx::pdl_enter();
+    __shared__ unsigned act_s[TW][kMaskWords];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int k = sat.k, nw = words_of(k);
+    const int X0 = ((int)blockIdx.x * TW + wi) * 32;
+    if (X0 >= WO) return;
+    const int Y0 = min((int)blockIdx.y * TY, HO - TY);
+    const int xe = min(X0 + 31, WO - 1), xl = min(X0 + lane, WO - 1);
+    const size_t down = (size_t)k * sat.P;                   // one image row further
+    unsigned *act = act_s[wi];
+    float hs[TY];
+#pragma unroll
+    for (int r = 0; r < TY; ++r) hs[r] = 0.f;
+    for (int f = 0; f < bs.F; ++f) {
+        const int32_t *tc = tcounts + (size_t)f * k;
+        int bx0 = 1 << 30, by0 = 1 << 30, bx1 = 0, by1 = 0;  // the filter's bounding box
+        for (int q = bs.rect_begin[f]; q < bs.rect_begin[f + 1]; ++q) {
+            bx0 = min(bx0, bs.rect[q].x0), by0 = min(by0, bs.rect[q].y0);
+            bx1 = max(bx1, bs.rect[q].x1), by1 = max(by1, bs.rect[q].y1);
+        }
+        __syncwarp();                                        // the words of the filter before are read
+        visit_words<T>(act, k, testable<T>(bx1 - bx0 + 31, by1 - by0 + TY - 1),
+                       Region<T>(sat, X0 + bx0, Y0 + by0, xe + bx1, Y0 + TY - 1 + by1));
+        __syncwarp();
+        long long ts = 0, acc[TY];
+        for (int j = 0; j < k; ++j) ts += abs(tc[j]);
+#pragma unroll
+        for (int r = 0; r < TY; ++r) acc[r] = ts;
+        int w = 0;
+        unsigned m = act[0];
+        while (true) {
+            while (m == 0 && ++w < nw) m = act[w];
+            if (m == 0) break;
+            const int j = word_cluster(w, m), t = tc[j];
+            m &= m - 1;
+            const T *base = sat.S + ((size_t)Y0 * k + j) * sat.P + xl;
+            int v[TY];
+#pragma unroll
+            for (int r = 0; r < TY; ++r) v[r] = 0;
+            for (int q = bs.rect_begin[f]; q < bs.rect_begin[f + 1]; ++q) {
+                const RectSpec &rc = bs.rect[q];
+                const T *top = base + rc.y0 * down, *bot = base + rc.y1 * down;
+#pragma unroll
+                for (int r = 0; r < TY; ++r)
+                    v[r] += rc.weight * box<T>(bot[r * down + rc.x1], bot[r * down + rc.x0], top[r * down + rc.x1],
+                                               top[r * down + rc.x0]);
+            }
+#pragma unroll
+            for (int r = 0; r < TY; ++r) acc[r] += abs(t - v[r]) - abs(t);
+        }
+#pragma unroll
+        for (int r = 0; r < TY; ++r) hs[r] = fmaf(bs.coef[f], (float)acc[r], hs[r]);
+    }
+    warp_argmax(put_tile<TY>(hs, X0 + lane, Y0, WO, heat, 0ull), amax);
+}
+
+// Cost of the tile kernel less that of the dense kernel, over a sample of 64 x 4 tiles: in
+// hundredths of a nanosecond on the full GPU, a visited pair costs 27 (0.244 to 0.307 ns measured
+// at 2048 x 2048 on random and on coherent labels), and in the dense kernel a cluster 25 and each
+// of its template-present pairs 10 (1.13 ms for 14,400 tiles of 128 clusters with 3.8 pairs each).
+// One warp per (sampled tile, slot).  The warps of the first tile also leave their slot's template
+// side: its counts in rows of 256, and the sum of the positive ones.
+template <typename T>
+__global__ void __launch_bounds__(128) score_probe_kernel(Sat<T> sat, int HO, int WO, int ntx, int nsample, int step,
+                                                          GridSpec gs, unsigned test, const int32_t *__restrict__ tcounts,
+                                                          ScoreAux *aux)
+{
+    ptx::pdl_enter();
+    const int lane = threadIdx.x & 31, k = sat.k, nslot = gs.G * gs.G + gs.full;
+    const int id = blockIdx.x * 4 + (threadIdx.x >> 5), q = id % nslot, i = id / nslot;
+    if (i >= nsample) return;
+    const long long tile = (long long)i * step;
+    const int X0 = (int)(tile % ntx) * 64, Y0 = min((int)(tile / ntx) * 4, HO - 4), xe = min(X0 + 63, WO - 1);
+    const Slot sl(gs, q);
+    const Region<T> reg(sat, X0 + sl.x0, Y0 + sl.y0, xe + sl.x1, Y0 + 3 + sl.y1);
+    const int32_t *tc = tcounts + (size_t)gs.slot_filter[q] * k;
+    int present = 0, visited = 0, ts = 0;
+    for (int j0 = 0; j0 < k; j0 += 128) {
+        const int j = j0 + 4 * lane;
+        const unsigned h = j >= k ? 0u : (test >> q) & 1 ? reg.holds4(j) : 15u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = j + u < k ? tc[j + u] : 0;
+            ts += max(t, 0);
+            present += t > 0;
+            visited += t > 0 && ((h >> u) & 1u);
+            if (i == 0) aux->t[q][j + u] = t;
+        }
+    }
+    const int d = __reduce_add_sync(0xffffffffu, 27 * visited - 10 * present);
+    ts = __reduce_add_sync(0xffffffffu, ts);
+    if (lane == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&aux->probe), (unsigned long long)(long long)d);
+        if (i == 0) aux->tsum[q] = ts;
+    }
+}
+
+// Slots whose region, swept over a tile of w x h windows, is tested.
+template <typename T>
+unsigned slot_tests(const GridSpec &gs, int w, int h)
+{
+    unsigned test = 0;
+    for (int q = 0; q <= gs.G * gs.G; ++q) {
+        const bool full = q == gs.G * gs.G;
+        const int sw = full ? gs.bx[gs.G] : gs.bx[q % gs.G + 1] - gs.bx[q % gs.G];
+        const int sh = full ? gs.by[gs.G] : gs.by[q / gs.G + 1] - gs.by[q / gs.G];
+        test |= (unsigned)testable<T>(sw + w - 1, sh + h - 1) << q;
+    }
+    return test;
+}
+
+template <typename T>
+cudaError_t launch_wgrid(const Sat<T> &sat, int HO, int WO, const WGridSpec &ws, const int32_t *tc, float *heat,
+                         unsigned long long *amax, cudaStream_t s)
+{
+    unsigned test = 0;
+    int w = 0;
+    bool sep = true;
+    for (int g = 0; g < ws.NG; ++g) {
+        const int gw = ws.bx[g][3] - ws.bx[g][0];
+        w = gw > w ? gw : w;
+        sep = sep && ws.sep[g];
+        test |= (unsigned)testable<T>(gw + 32 * kWX - 1, ws.by[g][3] - ws.by[g][0] + kWY - 1) << g;
+    }
+    const int nch = WTile<T>::chunks(w);
+    const size_t smem = TW * WNST * WTile<T>::stage(nch);
+    auto kernel = sep ? score_wgrid_tile_kernel<T, true> : score_wgrid_tile_kernel<T, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3((WO + 32 * kWX * TW - 1) / (32 * kWX * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), smem, s, sat,
+                      HO, WO, ws, test, nch, tc, heat, amax);
+}
+
+template <typename T>
+Sat<T> make_sat(const void *S, const void *coarse, int W, int k)
+{
+    return Sat<T>{static_cast<const T *>(S), static_cast<const T *>(coarse), sat_pitch(W), k, sat_coarse_cols(W),
+                  sat_coarse_pitch(k)};
+}
+
+template <typename T>
+cudaError_t launch_tiles_t(const Sat<T> &sat, int HO, int WO, const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws,
+                           const int32_t *tc, float *heat, ScoreAux *aux, long long dense_from, cudaStream_t s)
+{
+    unsigned long long *amax = &aux->amax;
+    if (gs.G > 0)
+        return launch_pdl(score_grid_tile_kernel<T, 2, kGridY>, dim3((WO + 64 * TW - 1) / (64 * TW), (HO + kGridY - 1) / kGridY), dim3(32 * TW),
+                          0, s, sat, HO, WO, gs, slot_tests<T>(gs, 64, kGridY), heat, aux, dense_from);
+    if (HO >= kWY) {
+        if (ws.NG > 0) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
+        return launch_pdl(score_generic_kernel<T, 4>, dim3((WO + 32 * TW - 1) / (32 * TW), (HO + 3) / 4), dim3(32 * TW), 0, s,
+                          sat, HO, WO, bs, tc, heat, amax);
+    }
+    return launch_pdl(score_generic_kernel<T, 1>, dim3((WO + 32 * TW - 1) / (32 * TW), HO), dim3(32 * TW), 0, s, sat, HO, WO,
+                      bs, tc, heat, amax);
+}
+
+}  // namespace
+
+// The tile kernel needs whole tiles and 32-bit offsets between a tile's rows.  Below 512 tiles (a
+// 256 x 256 query: 16 us dense, 24 us in tiles) a tile's chain of pairs is longer than the dense
+// kernel's whole run, and with at most 16 clusters nearly every cluster is in every window
+// (1019 x 972, k = 8: 38 us dense, 60 us in tiles); both stay dense without a probe.
+ScoreRoute score_grid_route(int HO, int WO, int k, int P, int th)
+{
+    const long long tiles = (long long)((WO + 63) / 64) * ((HO + 3) / 4);
+    const bool far = (long long)(th + 4) * k * (P / 4) >= (1ll << 32);
+    return HO < 4 || k <= 16 || tiles < 512 || far ? kScoreDense : kScoreProbe;
+}
+
+cudaError_t launch_score_probe(const void *coarse, bool u16, int W, int k, int HO, int WO, const GridSpec &gs,
+                               const int32_t *tc, ScoreAux *aux, long long *dense_from, cudaStream_t s)
+{
+    const int ntx = (WO + 63) / 64, nslot = gs.G * gs.G + gs.full;
+    const long long ntile = (long long)ntx * ((HO + 3) / 4);
+    const int step = (int)(ntile / 509 > 1 ? (ntile / 509) | 1 : 1);      // about 500 tiles
+    const int n = (int)((ntile + step - 1) / step);
+    *dense_from = 25ll * k * n;
+    const dim3 grid((unsigned)((n * nslot + 3) / 4)), block(128);
+    return u16 ? launch_pdl(score_probe_kernel<uint16_t>, grid, block, 0, s, make_sat<uint16_t>(nullptr, coarse, W, k), HO, WO,
+                            ntx, n, step, gs, slot_tests<uint16_t>(gs, 64, 4), tc, aux)
+               : launch_pdl(score_probe_kernel<uint32_t>, grid, block, 0, s, make_sat<uint32_t>(nullptr, coarse, W, k), HO, WO,
+                            ntx, n, step, gs, slot_tests<uint32_t>(gs, 64, 4), tc, aux);
+}
+
+cudaError_t launch_score_tiles(const void *S, const void *coarse, bool u16, int W, int k, int HO, int WO,
+                               const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
+                               ScoreAux *aux, long long dense_from, cudaStream_t s)
+{
+    return u16 ? launch_tiles_t(make_sat<uint16_t>(S, coarse, W, k), HO, WO, bs, gs, ws, tc, heat, aux, dense_from, s)
+               : launch_tiles_t(make_sat<uint32_t>(S, coarse, W, k), HO, WO, bs, gs, ws, tc, heat, aux, dense_from, s);
+}
+
+}  // namespace vqnnf
