@@ -148,14 +148,19 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint8_
 }
 
 // The pixels of cluster j in increasing order, written to out[0, cnt_j): a block-wide stable
-// compaction of the labels (for the in-order FP64 route only).  scan: blockDim.x ints of
-// shared memory.  Every thread of the block must call it.
+// compaction of the labels (for the in-order FP64 route only), four labels per load (lab is
+// 256-byte aligned).  scan: blockDim.x ints of shared memory.  Every thread of the block must call
+// it.
 __device__ void ordered_members(const uint8_t *__restrict__ lab, int l, int j, int *out, int *scan)
 {
     const int nt = blockDim.x, t = threadIdx.x;
-    const int seg = (l + nt - 1) / nt, p0 = min(l, t * seg), p1 = min(l, p0 + seg);
+    const int words = l >> 2, seg = (words + nt - 1) / nt, q0 = min(words, t * seg), q1 = min(words, q0 + seg);
+    const uint32_t *lab4 = reinterpret_cast<const uint32_t *>(lab);
+    const uint32_t jj = (uint32_t)j * 0x01010101u;
     int n = 0;
-    for (int p = p0; p < p1; ++p) n += lab[p] == j;
+    for (int q = q0; q < q1; ++q) n += __popc(__vcmpeq4(__ldg(lab4 + q), jj)) >> 3;
+    if (t == nt - 1)                                     // the last thread also takes the byte tail
+        for (int p = 4 * words; p < l; ++p) n += lab[p] == j;
     scan[t] = n;
     __syncthreads();
     for (int o = 1; o < nt; o <<= 1) {                   // inclusive scan (Hillis-Steele)
@@ -165,9 +170,75 @@ __device__ void ordered_members(const uint8_t *__restrict__ lab, int l, int j, i
         __syncthreads();
     }
     int pos = scan[t] - n;
-    for (int p = p0; p < p1; ++p)
-        if (lab[p] == j) out[pos++] = p;
+    for (int q = q0; q < q1; ++q) {
+        const uint32_t e = __vcmpeq4(__ldg(lab4 + q), jj);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (e >> (8 * c) & 1u) out[pos++] = 4 * q + c;
+    }
+    if (t == nt - 1)
+        for (int p = 4 * words; p < l; ++p)
+            if (lab[p] == j) out[pos++] = p;
     __syncthreads();
+}
+
+// The FP64 sum of Tc[m[0] D], Tc[m[1] D], .. (n values, one column of the members in pixel order),
+// added one by one in that order: one warp, the same result in every lane.
+//
+// The values are taken 64 at a time.  All of them, and the running sum s, are multiples of 2^g, g the
+// smaller of the last mantissa bit of the smallest nonzero value and the lowest set bit of s.  While
+// |s| + 64 max |x| < 2^(g + 53), every partial sum of the in-order evaluation is a multiple of 2^g
+// below 2^(g + 53), an FP64 number: no addition rounds, and s plus the exact sum of the 64 is what
+// the in-order evaluation gives.  That sum is taken in units of 2^-50 (a value below 2^-27 or at
+// least 2^6 is left out of it) over the lanes in 64-bit integers.  Where the test fails (a value with
+// bits below the last place of s, or s reaching its next power of two with its lowest bits in use;
+// rare), the 64 are added one by one.
+//
+// Latency-bound: adding value by value, a chain of n FP64 additions, took 92 us per update over ten
+// templates of up to 136 x 182 pixels, D = 256, 8 to 256 clusters (launch list); this takes 26 us.
+__device__ double in_order_sum(const float *__restrict__ Tc, const int *m, int n, int D)
+{
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    auto load = [&](int q) { return q < n ? __ldg(Tc + (size_t)m[q] * D) : 0.f; };
+    float n0 = load(lane), n1 = load(lane + 32);
+    for (int q = 0; q < n; q += 64) {
+        const float x0 = n0, x1 = n1;
+        n0 = load(q + 64 + lane);
+        n1 = load(q + 96 + lane);
+        const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
+        const int e0 = b0 >> 23 & 255, e1 = b1 >> 23 & 255;
+        const bool z0 = (b0 << 1) == 0u, z1 = (b1 << 1) == 0u;
+        const bool ok = (z0 || (e0 >= 100 && e0 <= 132)) && (z1 || (e1 >= 100 && e1 <= 132));
+        bool exact = __all_sync(0xffffffffu, ok);
+        if (exact) {
+            const int lo = __reduce_min_sync(0xffffffffu, min(z0 ? 255 : e0, z1 ? 255 : e1));
+            if (lo == 255) continue;                      // only zeros
+            const int hi = __reduce_max_sync(0xffffffffu, max(z0 ? 0 : e0, z1 ? 0 : e1));
+            // below 2^56 units each, 2^62 for 64 of them
+            long long f0 = z0 ? 0ll : (long long)(b0 & 0x7FFFFFu | 0x800000u) << (e0 - 100 & 63);
+            long long f1 = z1 ? 0ll : (long long)(b1 & 0x7FFFFFu | 0x800000u) << (e1 - 100 & 63);
+            f0 = (b0 >> 31 ? -f0 : f0) + (b1 >> 31 ? -f1 : f1);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) f0 += __shfl_xor_sync(0xffffffffu, f0, o);
+            int g = lo - 150;
+            const unsigned long long sb = (unsigned long long)__double_as_longlong(s);
+            if (sb << 1) {
+                const unsigned long long ms = (sb & 0xFFFFFFFFFFFFFull) | 1ull << 52;
+                g = min(g, (int)(sb >> 52 & 2047) - 1075 + __ffsll((long long)ms) - 1);
+            }
+            // |s| + 64 * 2^(hi - 126); rounding it cannot take it below a power of two that it reaches
+            const double top = fabs(s) + __longlong_as_double((long long)(hi - 126 + 6 + 1023) << 52);
+            const int et = (int)((unsigned long long)__double_as_longlong(top) >> 52 & 2047) - 1023;
+            exact = et < g + 53;
+            if (exact) s += (double)f0 * 0x1p-50;         // f0 is a multiple of 2^(g + 50) below 2^(g + 103)
+        }
+        if (!exact) {                                     // the padding adds +0
+            for (int r = 0; r < 32; ++r) s += (double)__shfl_sync(0xffffffffu, x0, r);
+            for (int r = 0; r < 32; ++r) s += (double)__shfl_sync(0xffffffffu, x1, r);
+        }
+    }
+    return s;
 }
 
 // c_j[i] = fl32( (sum over members, pixel order, FP64) / count ); empty clusters keep c_j.
@@ -258,8 +329,6 @@ __device__ __forceinline__ int top_bit(unsigned __int128 v)
     return hi ? 127 - __clzll((long long)hi) : (lo ? 63 - __clzll((long long)lo) : -1);
 }
 
-constexpr int FCH = 44;      // member rows per staged chunk of the in-order FP64 route
-
 // RN(a / b) for finite a and b > 0 from y = RN(1 / b) (Markstein's theorem: if q is within one
 // ulp of a / b, r = a - b q is exact and RN(q + r y) is the correctly rounded quotient).  The
 // first correction brings q0 = RN(a y), within 1.5 ulp, to within one ulp.
@@ -278,13 +347,12 @@ __global__ void __launch_bounds__(32 * UW, 5) update_kernel(const float *__restr
 {
     ptx::pdl_enter();
     __shared__ int sscan[32 * UW];
-    // the per-warp partial sums, later reused for the staged member values of the FP64 route
+    // the per-warp partial sums, later reused for the FP64 route's results
     __shared__ __align__(16) unsigned __int128 sacc[3][UW][32];
     __shared__ int slow[UW][32], shish[UW][32];
     __shared__ unsigned char sbad[UW][32];
     __shared__ unsigned s_need;
     __shared__ int s_last;
-    static_assert(2 * FCH * 33 * sizeof(float) <= sizeof(sacc), "staging buffers exceed the reused space");
     auto spos = sacc[0], sneg = sacc[1], smag = sacc[2];
     // (first slot, rows | cluster << 8, cluster's first chunk, cluster size); rows = 0: unused
     const int4 ch = lw.chunks[blockIdx.x];
@@ -446,30 +514,19 @@ __global__ void __launch_bounds__(32 * UW, 5) update_kernel(const float *__restr
         s = (negative ? -v : v) * __longlong_as_double((long long)(low - 80 + 1023) << 52);
     }
     if (nm) {
-        // the in-order FP64 sum of the flagged columns over all c members: the members are
-        // listed in pixel order, then the block's 32 columns of their rows are staged in shared
-        // memory, FCH rows at a time and double-buffered; warps 1..UW-1 load the next chunk
-        // while warp 0 adds the current one, row by row, in pixel order
+        // the in-order FP64 sum of the flagged columns over all c members, one warp per column
         int *mc = lw.ordered + lw.off[j];
         ordered_members(lab, l, j, mc, sscan);
-        float (*vals)[FCH][33] = reinterpret_cast<float (*)[FCH][33]>(&sacc[0][0][0]);
-        auto stage = [&](int q0, int buf, int w0, int nwarp) {
-            const int nrow = min(FCH, c - q0);
-            for (int r = w - w0; r < nrow; r += nwarp) vals[buf][r][lane] = __ldg(T + (size_t)mc[q0 + r] * D + ic);
-        };
-        stage(0, 0, 0, UW);
-        __syncthreads();
-        const bool mine = w == 0 && ((nm >> lane) & 1u);
-        double acc = 0.0;
-        for (int q0 = 0, t = 0; q0 < c; q0 += FCH, ++t) {
-            if (w != 0 && q0 + FCH < c) stage(q0 + FCH, (t + 1) & 1, 1, UW - 1);
-            if (mine) {
-                const int nrow = min(FCH, c - q0);
-                for (int r = 0; r < nrow; ++r) acc += (double)vals[t & 1][r][lane];
+        double *sres = reinterpret_cast<double *>(&sacc[0][0][0]);
+        int col = 0;
+        for (unsigned r = nm; r; r &= r - 1, ++col)
+            if (col % UW == w) {
+                const int cl = __ffs((int)r) - 1;
+                const double v = in_order_sum(T + blockIdx.y * 32 + cl, mc, c, D);
+                if (lane == 0) sres[cl] = v;
             }
-            __syncthreads();
-        }
-        if (mine) s = acc;
+        __syncthreads();
+        if (w == 0 && ((nm >> lane) & 1u)) s = sres[lane];
     }
     if (w == 0 && i < D) C[(size_t)j * D + i] = (float)(isfinite(s) ? div_rn(s, (double)c, __ldg(lw.rcp + j)) : s / (double)c);
 }
