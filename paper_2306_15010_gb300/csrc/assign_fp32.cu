@@ -244,10 +244,14 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
 }
 
 // ----------------------------------------------------------------------------------
-// FP32 SIMT contraction: 128 pixels x 128 centroids per pass, 8 x 8 outputs per thread,
+// FP32 SIMT contraction: 16 TM pixels x 16 TN centroids per pass, TM x TN outputs per thread,
 // sequential FMA accumulation over D (so the per-dot error is <= gamma_D sum |x c|).
+// Bound by the FMA pipe: packed FMAs on two outputs' lanes take 0.82 ms for 262,144 pixels, D = 512,
+// k = 128 (21 T FMA/s; scalar FMAs 1.00 ms).  Tiles of 8 x 4 take the same, 16 x 8 outputs or a step
+// of 8 dimensions 0.84 and 0.86 ms; the pixels' values stored twice, to load them as pairs, 1.02 ms
+// (the loads' 128 bytes per cycle bind).
 // ----------------------------------------------------------------------------------
-constexpr int BM = 128, BN = 128, BK = 16, NT = 256;
+constexpr int BK = 16, NT = 256;
 
 __device__ __forceinline__ void push_flag(bool flagged, unsigned int pix, const unsigned *mask,
                                           FlagList fl)
@@ -300,22 +304,62 @@ __device__ __forceinline__ int decide_pixel(const float *srow, int stride, int k
     return cnt == 1 ? last : amin;
 }
 
-__global__ void __launch_bounds__(NT, 2) assign_fp32_kernel(const float *__restrict__ X, long long n,
-                                                         int D, int k, CodebookPrep p,
-                                                         uint8_t *__restrict__ labels, FlagList fl)
+// The tile of a block: 16 x 16 threads of TM x TN outputs each.
+template <int TM, int TN>
+struct SimtTile {
+    static constexpr int BM = 16 * TM, BN = 16 * TN;
+    static constexpr int AP = BM + 4, BP = BN + 4;     // staged row pitches (conflict-free stores)
+    static constexpr int kStage = 2 * BK * (AP + BP);  // floats, double-buffered
+    static int kpad(int k) { return (k + BN - 1) / BN * BN; }
+    // one pass over the centroids: the scores reuse the staging buffers
+    static size_t smem(int k)
+    {
+        const size_t sc = (size_t)BM * (kpad(k) + 1), st = kStage;
+        return sizeof(float) * ((kpad(k) == BN ? (sc > st ? sc : st) : sc + st) + 4 * (size_t)kpad(k) + 4 * BM);
+    }
+};
+
+// A thread's N values of a staged row: N = 2 or 4 consecutive floats, or quads 64 apart.
+template <int N>
+__device__ __forceinline__ void lds_vec(float (&v)[N], const float *p)
 {
+    if constexpr (N == 2) {
+        const float2 a = *reinterpret_cast<const float2 *>(p);
+        v[0] = a.x, v[1] = a.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const float4 a = *reinterpret_cast<const float4 *>(p + 64 * q);
+            v[4 * q] = a.x, v[4 * q + 1] = a.y, v[4 * q + 2] = a.z, v[4 * q + 3] = a.w;
+        }
+    }
+}
+// Place inside a tile of 16 N of output i of thread t
+template <int N>
+__device__ __forceinline__ int tile_pos(int t, int i)
+{
+    return N > 4 ? (i / 4) * 64 + t * 4 + i % 4 : t * N + i;
+}
+
+template <int TM, int TN, int MB>
+__global__ void __launch_bounds__(NT, MB) assign_fp32_kernel(const float *__restrict__ X, long long n,
+                                                                       int D, int k, CodebookPrep p,
+                                                                       uint8_t *__restrict__ labels, FlagList fl)
+{
+    using L = SimtTile<TM, TN>;
+    constexpr int BM = L::BM, BN = L::BN;
     ptx::pdl_enter();
     extern __shared__ __align__(16) float smem[];
     const int kp = (k + BN - 1) / BN * BN;
     const int sp = kp + 1;
-    float *As = smem;                  // [2][BK][BM]
-    float *Bs = As + 2 * BK * BM;      // [2][BK][BN]
-    float *Sc = Bs + 2 * BK * BN;      // [BM][sp]
-    float *ca = Sc + BM * sp;          // [kp]
-    float *cv = ca + kp;
+    float *As = smem;                          // [2][BK][AP]
+    float *Bs = As + 2 * BK * L::AP;           // [2][BK][BP]
+    float *Sc = kp == BN ? smem : Bs + 2 * BK * L::BP;   // [BM][sp], over the staging buffers after a single pass
+    float *ca = kp == BN ? smem + (BM * sp > L::kStage ? BM * sp : L::kStage) : Sc + BM * sp;
+    float *cv = ca + kp;                       // [kp] each
     float *cb = cv + kp;
     float *cn = cb + kp;
-    float *xn = cn + kp;               // [2][BM]
+    float *xn = cn + kp;                       // [4][BM]
 
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
@@ -328,104 +372,115 @@ __global__ void __launch_bounds__(NT, 2) assign_fp32_kernel(const float *__restr
         cb[j] = ok ? p.b[jc] : 0.f;
         cn[j] = ok ? p.nrm[jc] : 0.f;
     }
-    // loader mapping: row lp (pixel or centroid), dims lh*8 .. lh*8+7 of the k-step
-    const int lp = tid >> 1, lh = tid & 1;
-    const long long prow = p0 + lp;
-    const bool prow_ok = prow < n;
-    const float *xrow = X + (prow_ok ? prow : 0) * (long long)D;
-    float xsq = 0.f;
+    // loader mapping: row tid / LQ + LR u (pixel or centroid), dims 4 (tid % LQ) .. + 3 of the k-step
+    constexpr int LQ = BK / 4, LR = NT / LQ, LA = (BM + LR - 1) / LR, LB = (BN + LR - 1) / LR;
+    const int lr = tid / LQ, lq = tid % LQ;
+    const bool ahas = BM >= LR || lr < BM, bhas = BN >= LR || lr < BN;
+    float xsq[LA];
+#pragma unroll
+    for (int u = 0; u < LA; ++u) xsq[u] = 0.f;
 
     for (int nc = 0; nc < kp; nc += BN) {
-        const int crow = nc + lp;
-        const bool crow_ok = crow < k;
-        const float *crw = p.cc + (size_t)(crow_ok ? crow : 0) * D;
-        float acc[8][8];
+        // pairs of centroids side by side: one packed FMA per two outputs, each component
+        // rounded as the scalar FMA (the sums over D stay sequential)
+        float2 acc[TM][TN / 2];
 #pragma unroll
-        for (int a = 0; a < 8; ++a)
+        for (int a = 0; a < TM; ++a)
 #pragma unroll
-            for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+            for (int b = 0; b < TN / 2; ++b) acc[a][b] = make_float2(0.f, 0.f);
 
-        float ra[8], rb[8];
+        float4 ra[LA], rb[LB];
         // Every load address is clamped into its buffer and out-of-range values are
         // zeroed afterwards: no address past a buffer is ever formed, even for loads the
         // compiler may issue ahead of their guard.
         auto gload = [&](int d0) {
+            const int d = d0 + lq * 4;
+            const bool din = d < D;
+            const int dc = din ? d : D - 4;
+            const float4 mm = __ldg(reinterpret_cast<const float4 *>(p.mean + dc));
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int d = d0 + lh * 8 + q * 4;
-                const bool din = d < D;
-                const int dc = din ? d : D - 4;
-                float4 xa = __ldg(reinterpret_cast<const float4 *>(xrow + dc));
-                const float4 mm = __ldg(reinterpret_cast<const float4 *>(p.mean + dc));
-                float4 cbv = __ldg(reinterpret_cast<const float4 *>(crw + dc));
-                const bool xok = din && prow_ok, cok = din && crow_ok;
-                xa.x = xok ? xa.x - mm.x : 0.f; xa.y = xok ? xa.y - mm.y : 0.f;
-                xa.z = xok ? xa.z - mm.z : 0.f; xa.w = xok ? xa.w - mm.w : 0.f;
-                cbv.x = cok ? cbv.x : 0.f; cbv.y = cok ? cbv.y : 0.f;
-                cbv.z = cok ? cbv.z : 0.f; cbv.w = cok ? cbv.w : 0.f;
-                ra[q * 4 + 0] = xa.x; ra[q * 4 + 1] = xa.y; ra[q * 4 + 2] = xa.z; ra[q * 4 + 3] = xa.w;
-                rb[q * 4 + 0] = cbv.x; rb[q * 4 + 1] = cbv.y; rb[q * 4 + 2] = cbv.z; rb[q * 4 + 3] = cbv.w;
+            for (int u = 0; u < LA; ++u) {
+                const long long pr = p0 + lr + LR * u;
+                const bool ok = din && ahas && pr < n;
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(X + (pr < n ? pr : 0) * (long long)D + dc));
+                ra[u] = ok ? make_float4(v.x - mm.x, v.y - mm.y, v.z - mm.z, v.w - mm.w) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < LB; ++u) {
+                const int cr = nc + lr + LR * u;
+                const bool ok = din && bhas && cr < k;
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(p.cc + (size_t)(cr < k ? cr : 0) * D + dc));
+                rb[u] = ok ? v : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         };
         auto sstore = [&](int buf) {
-            float *a = As + buf * BK * BM;
-            float *b = Bs + buf * BK * BN;
+            float *a = As + buf * BK * L::AP + lq * 4 * L::AP + lr;
+            float *b = Bs + buf * BK * L::BP + lq * 4 * L::BP + lr;
+            if (ahas)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                a[(lh * 8 + q) * BM + lp] = ra[q];
-                b[(lh * 8 + q) * BN + lp] = rb[q];
-            }
+                for (int u = 0; u < LA; ++u) {
+                    const float v[4] = {ra[u].x, ra[u].y, ra[u].z, ra[u].w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        a[q * L::AP + LR * u] = v[q];
+                        if (nc == 0) xsq[u] = fmaf(v[q], v[q], xsq[u]);
+                    }
+                }
+            if (bhas)
+#pragma unroll
+                for (int u = 0; u < LB; ++u) {
+                    b[LR * u] = rb[u].x;
+                    b[L::BP + LR * u] = rb[u].y;
+                    b[2 * L::BP + LR * u] = rb[u].z;
+                    b[3 * L::BP + LR * u] = rb[u].w;
+                }
         };
         gload(0);
-        if (nc == 0)
-#pragma unroll
-            for (int q = 0; q < 8; ++q) xsq = fmaf(ra[q], ra[q], xsq);
         sstore(0);
         __syncthreads();
         int buf = 0;
         for (int d0 = 0; d0 < D; d0 += BK) {
             const bool more = d0 + BK < D;
             if (more) gload(d0 + BK);   // gload clamps its addresses
-            const float *a = As + buf * BK * BM;
-            const float *b = Bs + buf * BK * BN;
+            const float *a = As + buf * BK * L::AP + ty * (TM > 4 ? 4 : TM);
+            const float *b = Bs + buf * BK * L::BP + tx * (TN > 4 ? 4 : TN);
 #pragma unroll
             for (int kk = 0; kk < BK; ++kk) {
-                const float4 a0 = *reinterpret_cast<const float4 *>(a + kk * BM + ty * 4);
-                const float4 a1 = *reinterpret_cast<const float4 *>(a + kk * BM + 64 + ty * 4);
-                const float4 b0 = *reinterpret_cast<const float4 *>(b + kk * BN + tx * 4);
-                const float4 b1 = *reinterpret_cast<const float4 *>(b + kk * BN + 64 + tx * 4);
-                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                float av[TM], bv[TN];
+                lds_vec<TM>(av, a + kk * L::AP);
+                lds_vec<TN>(bv, b + kk * L::BP);
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < TM; ++i) {
+                    const float2 aa = make_float2(av[i], av[i]);
 #pragma unroll
-                    for (int jj = 0; jj < 8; ++jj) acc[i][jj] = fmaf(av[i], bv[jj], acc[i][jj]);
+                    for (int jj = 0; jj < TN / 2; ++jj)
+                        acc[i][jj] = __ffma2_rn(aa, make_float2(bv[2 * jj], bv[2 * jj + 1]), acc[i][jj]);
+                }
             }
-            if (more) {
-                if (nc == 0)
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) xsq = fmaf(ra[q], ra[q], xsq);
-                sstore(buf ^ 1);
-            }
+            if (more) sstore(buf ^ 1);
             __syncthreads();
             buf ^= 1;
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = (i < 4) ? ty * 4 + i : 64 + ty * 4 + (i - 4);
+        for (int i = 0; i < TM; ++i) {
+            const int r = tile_pos<TM>(ty, i);
 #pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-                const int c = nc + ((jj < 4) ? tx * 4 + jj : 64 + tx * 4 + (jj - 4));
-                Sc[r * sp + c] = fmaf(-2.0f, acc[i][jj], cn[c]);
+            for (int jj = 0; jj < TN; ++jj) {
+                const int c = nc + tile_pos<TN>(tx, jj);
+                Sc[r * sp + c] = fmaf(-2.0f, jj & 1 ? acc[i][jj / 2].y : acc[i][jj / 2].x, cn[c]);
             }
         }
     }
-    xn[lh * BM + lp] = xsq;
+    if (ahas)
+#pragma unroll
+        for (int u = 0; u < LA; ++u) xn[lq * BM + lr + LR * u] = xsq[u];
     __syncthreads();
     if (tid < BM) {
         const long long pix = p0 + tid;
         const bool valid = pix < n;
-        const float xs = xn[tid] + xn[BM + tid];
+        float xs = 0.f;
+#pragma unroll
+        for (int q = 0; q < LQ; ++q) xs += xn[q * BM + tid];
         const float X = sqrtf(xs) * (1.0f + (float)(D + 8) * (float)kU32);
         unsigned mask[kMaskWords];
         int ncand = 1;
@@ -644,25 +699,35 @@ cudaError_t launch_prep_codebook(const float *C, int k, int D, int prec, Codeboo
     return cudaGetLastError();
 }
 
-static size_t fp32_smem_bytes(int k)
+template <int TM, int TN, int MB>
+static cudaError_t launch_simt(const float *X, long long n, int D, int k, const CodebookPrep &p, uint8_t *labels,
+                               FlagList fl, cudaStream_t s)
 {
-    const int kp = (k + BN - 1) / BN * BN;
-    return sizeof(float) * (size_t)(2 * BK * BM + 2 * BK * BN + BM * (kp + 1) + 4 * kp + 2 * BM);
+    using L = SimtTile<TM, TN>;
+    const size_t smem = L::smem(k);
+    const cudaError_t e = cudaFuncSetAttribute(assign_fp32_kernel<TM, TN, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem);
+    if (e != cudaSuccess) return e;
+    const long long blocks = (n + L::BM - 1) / L::BM;
+    return launch_pdl(assign_fp32_kernel<TM, TN, MB>, dim3((unsigned)blocks), dim3(NT), smem, s, X, n, D, k, p, labels, fl);
 }
 
 cudaError_t launch_assign_fp32(const float *X, long long n, int D, int k, const CodebookPrep &p,
                                uint8_t *labels, FlagList fl, cudaStream_t s)
 {
-    const size_t smem = fp32_smem_bytes(k);
-    cudaError_t e = cudaFuncSetAttribute(assign_fp32_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const long long blocks = (n + BM - 1) / BM;
-    {
-        const cudaError_t le_ = launch_pdl(assign_fp32_kernel, dim3((unsigned)blocks), dim3(NT), smem, s, X, n, D, k, p, labels, fl);
-        if (le_ != cudaSuccess) return le_;
+    // Blocks of 32 pixels where 128-pixel ones would leave most SMs idle (1,024 pixels, D = 64,
+    // k = 16: 8.8 against 10.9 us; equal from 4,096 pixels on); the codebook's columns padded to 32,
+    // 64 or 128 (65,536 pixels, D = 64, k = 16: 19 us, padded to 128 39 us).  Codebooks of more than
+    // 128 centroids keep a pixel's scores of both passes (one block per SM whatever its registers).
+    if (n <= 4096) {
+        if (k <= 32) return launch_simt<2, 2, 4>(X, n, D, k, p, labels, fl, s);
+        if (k <= 64) return launch_simt<2, 4, 4>(X, n, D, k, p, labels, fl, s);
+        return launch_simt<2, 8, 4>(X, n, D, k, p, labels, fl, s);
     }
-    return cudaGetLastError();
+    if (k <= 32) return launch_simt<8, 2, 2>(X, n, D, k, p, labels, fl, s);
+    if (k <= 64) return launch_simt<8, 4, 2>(X, n, D, k, p, labels, fl, s);
+    if (k <= 128) return launch_simt<8, 8, 2>(X, n, D, k, p, labels, fl, s);
+    return launch_simt<8, 8, 1>(X, n, D, k, p, labels, fl, s);
 }
 
 cudaError_t launch_rescore(const float *X, long long n, int D, const float *C, int k,
