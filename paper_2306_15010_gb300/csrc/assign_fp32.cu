@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
         const float c = C[(size_t)j * D + i], m = p.mean[i];
         float cf, d32;
         two_sum(c, -m, cf, d32);                      // c - m = cf + d32 exactly
-        p.cc[(size_t)j * D + i] = cf;
+        if (prec != VQNNF_PREC_FP8) p.cc[(size_t)j * D + i] = cf;   // the FP8 path keeps a2 and v2 in its place
         const uint32_t hb = bf16_round_exact(cf, d32);
         const float hf = bf16_value(hb);
         float rf, rd;
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
         const double nhi = sqrt((double)tot[5] * up) * margin;
         const double nlo = sqrt((double)tot[6] * up) * margin;
         const double nd16 = sqrt((double)tot[7] * up) * margin;
-        double a, v;
+        double a = 0.0, v = 0.0;
         if (prec == VQNNF_PREC_FP32) {
             const double gD = (double)D * u / (1.0 - (double)D * u);
             a = 2.0 * gD * ncc + 2.0 * (1.0 + 2.0 * u) * nd32;
@@ -227,14 +227,21 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
             a = 2.0 * (dc + gacc * nq) * (1.0 + 4.0 * u);
             v = 2.0 * nc;
             p.csc[j] = csc;
-        } else {
+        }
+        if (prec != VQNNF_PREC_FP32) {
             // Three BF16 products x_hi.hi + x_hi.lo + x_lo.hi.  Tensor-core accumulation
             // order and rounding are not documented: take four times the sequential FP32
             // bound.  The x_lo terms (||x_lo|| <= 2^-8 ||x_hi||) are folded into a_j:
             //   |err| <= X [gacc (|hi| + |lo|) + |d|] + X_lo [gacc |hi| + |lo| + |d|] + ...
             const double gacc = (double)D * 4.0 * u;
-            a = 2.0 * (gacc * (nhi + nlo) + nd16) + 2.0 * 0.00390625 * (gacc * nhi + nlo + nd16);
-            v = 2.0 * nc;
+            const double a16 = 2.0 * (gacc * (nhi + nlo) + nd16) + 2.0 * 0.00390625 * (gacc * nhi + nlo + nd16);
+            if (prec == VQNNF_PREC_FP8) {
+                p.a2[j] = __double2float_ru(a16);
+                p.v2[j] = __double2float_ru(2.0 * nc);
+            } else {
+                a = a16;
+                v = 2.0 * nc;
+            }
         }
         p.nrm[j] = n32;
         p.a[j] = __double2float_ru(a);
@@ -529,13 +536,15 @@ constexpr int RS_MAXC = 16;        // 32-feature chunks of a pixel held in regis
 __global__ void __launch_bounds__(256, 2) rescore_kernel(const float *__restrict__ X, int D,
                                                       const float *__restrict__ C, int k,
                                                       uint8_t *__restrict__ labels, FlagList fl,
-                                                      unsigned cap)
+                                                      unsigned cap, SecondPass second)
 {
     ptx::pdl_enter();
     const int lane = threadIdx.x & 31;
     const unsigned wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned nw = (gridDim.x * blockDim.x) >> 5;
-    const unsigned n_entries = min(*fl.count, cap);     // the list holds at most cap entries
+    unsigned listed = *fl.count;
+    if (second.first && listed > second.limit) listed = *second.count;   // the second pass's list
+    const unsigned n_entries = min(listed, cap);        // the list holds at most cap entries
     const float u = (float)kU32;
     const float rho = ((float)((D + 31) / 32) + 8.0f) * u * 1.01f + 4.0f * u;
     unsigned long long my_cand = 0, my_deep = 0;
@@ -673,11 +682,11 @@ __global__ void __launch_bounds__(256, 2) rescore_kernel(const float *__restrict
     }
 }
 
-__global__ void finish_stats_kernel(FlagList fl, vqnnf_assign_stats *out)
+__global__ void finish_stats_kernel(FlagList fl, bool fp8, vqnnf_assign_stats *out)
 {
     ptx::pdl_enter();
     out->n_flagged = *fl.count;
-    out->n_candidates = fl.stats[1];
+    out->n_candidates = fp8 ? fl.stats[4] : fl.stats[1];   // of the pixels counted above
     out->n_deep = fl.stats[2];
     out->reserved = 0;
 }
@@ -731,7 +740,7 @@ cudaError_t launch_assign_fp32(const float *X, long long n, int D, int k, const 
 }
 
 cudaError_t launch_rescore(const float *X, long long n, int D, const float *C, int k,
-                           uint8_t *labels, FlagList fl, cudaStream_t s)
+                           uint8_t *labels, FlagList fl, cudaStream_t s, SecondPass second)
 {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
@@ -740,16 +749,16 @@ cudaError_t launch_rescore(const float *X, long long n, int D, const float *C, i
     // (the Lloyd steps' template assignments) launch fewer blocks
     const long long blocks = std::min<long long>((long long)sms * 8, std::max<long long>(sms, (n + 63) / 64));
     {
-        const cudaError_t le_ = launch_pdl(rescore_kernel, dim3((unsigned)blocks), dim3(256), 0, s, X, D, C, k, labels, fl, (unsigned)n);
+        const cudaError_t le_ = launch_pdl(rescore_kernel, dim3((unsigned)blocks), dim3(256), 0, s, X, D, C, k, labels, fl, (unsigned)n, second);
         if (le_ != cudaSuccess) return le_;
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_finish_stats(FlagList fl, vqnnf_assign_stats *out, cudaStream_t s)
+cudaError_t launch_finish_stats(FlagList fl, bool fp8, vqnnf_assign_stats *out, cudaStream_t s)
 {
     {
-        const cudaError_t le_ = launch_pdl(finish_stats_kernel, dim3(1), dim3(1), 0, s, fl, out);
+        const cudaError_t le_ = launch_pdl(finish_stats_kernel, dim3(1), dim3(1), 0, s, fl, fp8, out);
         if (le_ != cudaSuccess) return le_;
     }
     return cudaGetLastError();

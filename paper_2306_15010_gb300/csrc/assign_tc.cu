@@ -59,6 +59,7 @@ constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
 constexpr int PF = 0;              // chunks prefetched into L2 ahead of the loads (none: measured best)
 
 struct TcArgs {
+    SecondPass second;
     long long n;
     int D, krows, npad, nkc, sb, sf, nb, sa, pf;   // krows: rows of the prepared codebook
     long long ntiles;
@@ -265,6 +266,7 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
                                                           const __grid_constant__ TcArgs g)
 {
     ptx::pdl_enter();
+    if (g.second.first && *g.second.first <= g.second.limit) return;   // uniform over the grid
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int npad = g.npad, D = g.D, nkc = g.nkc, SB = g.sb, SF = g.sf, NB = g.nb, SA = g.sa;
@@ -1063,6 +1065,8 @@ __global__ void __launch_bounds__(F8_NT, 1) assign_fp8_kernel(const __grid_const
             const bool flagged = valid && cnt > 1;
             const unsigned ballot = __ballot_sync(0xffffffffu, flagged);
             if (ballot) {
+                const unsigned ncand = __reduce_add_sync(0xffffffffu, flagged ? (unsigned)cnt : 0u);
+                if (lane == 0) atomicAdd(&g.fl.stats[4], (unsigned long long)ncand);
                 const int leader = __ffs(ballot) - 1;
                 unsigned basei = 0;
                 if (lane == leader) basei = atomicAdd(g.fl.count, (unsigned)__popc(ballot));
@@ -1138,7 +1142,7 @@ size_t tc_smem_bytes(int npad, int D, int sb, int sf, int ncols = 0, int nsegcap
 }  // namespace
 
 cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const CodebookPrep &p, int krows,
-                                   const TcSeg *seg, int nseg, int sf_req, int pf, cudaStream_t s)
+                                   const TcSeg *seg, int nseg, int sf_req, int pf, cudaStream_t s, SecondPass second)
 {
     if (D % 16 != 0 || nseg < 1 || nseg > kMaxSeg || krows < 1 || n < 1) return cudaErrorNotSupported;
     int npad = 0;
@@ -1186,6 +1190,7 @@ cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const Cod
         return e;
     TcArgs a;
     memset(&a, 0, sizeof(a));
+    a.second = second;
     a.n = n;
     a.D = D;
     a.krows = krows;
@@ -1307,7 +1312,7 @@ cudaError_t launch_assign_bf16_stat(const float *X, long long n, int D, const Co
 }
 
 cudaError_t launch_assign_bf16(const float *X, long long n, int D, int k, const CodebookPrep &p,
-                               uint8_t *labels, FlagList fl, cudaStream_t s)
+                               uint8_t *labels, FlagList fl, cudaStream_t s, SecondPass second)
 {
     if (k < 1 || k > kMaxK) return cudaErrorNotSupported;
     TcSeg one;
@@ -1316,7 +1321,7 @@ cudaError_t launch_assign_bf16(const float *X, long long n, int D, int k, const 
     one.k = k;
     one.labels = labels;
     one.fl = fl;
-    return launch_assign_bf16_seg(X, n, D, p, k, &one, 1, 0, -1, s);
+    return launch_assign_bf16_seg(X, n, D, p, k, &one, 1, 0, -1, s, second);
 }
 
 bool fp8_supported(int D, int k)

@@ -98,7 +98,7 @@ struct BatchWs {
     unsigned *flcount;                        // kMaxSegStat x 64 (counters and stats, one memset)
     FlagList fl[kMaxSegStat];
     float *sC;                                // stationary codebooks, every launch's groups in a row
-    CodebookPrep sprep;                       // their prepared planes (one common centring mean)
+    CodebookPrep sprep = {};                  // their prepared planes (one common centring mean)
     FitWs fit[kLanes];                        // per lane: the k-means and template-NNF workspace
     char *score_base[kLanes];                 // integral-image workspace of one pair per lane
     float *heat_scratch[kLanes];              // heatmap of one pair when the caller wants maxima only
@@ -132,7 +132,7 @@ BatchWs carve_batch(WsCursor &c, const vqnnf_image *q, int nq, const vqnnf_batch
     }
     for (int g = 0; g < nt; ++g) {            // at most one group per template
         w.gC.push_back(c.take<float>((size_t)kGroupRows * D));
-        CodebookPrep p;
+        CodebookPrep p = {};
         p.mean = c.take<float>((size_t)D);
         p.cc = c.take<float>((size_t)kGroupRows * D);
         p.chi = c.take<uint16_t>((size_t)kGroupRows * D);

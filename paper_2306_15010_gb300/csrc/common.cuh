@@ -24,6 +24,7 @@ struct CodebookPrep {
     float *b;         // k       bound constant (error of nrm)
     uint8_t *cq8;     // k x D   FP8 e4m3 of (c_j - m) / s_j                 (FP8 path)
     float *csc;       // k       the power-of-two scale s_j                  (FP8 path)
+    float *a2, *v2;   // k       a and v of the BF16 contraction             (FP8 path, second pass)
 };
 
 // FP8 path: the features quantised per row (x - m = s_x q + residual, s_x a power of two).
@@ -37,7 +38,8 @@ struct FlagList {
     unsigned int *count;      // device counter
     unsigned int *pix;        // capacity entries
     unsigned int *mask;       // capacity x kMaskWords candidate bit sets
-    unsigned long long *stats;  // [n_flagged, n_candidates, n_deep, reserved]
+    unsigned long long *stats;  // [-, candidates re-scored, pixels of the double-float stage, -,
+                                //  candidates the FP8 contraction left]
 };
 
 // One codebook among several side by side in the columns of one tensor-core contraction:
@@ -61,9 +63,16 @@ cudaError_t launch_prep_codebook(const float *C, int k, int D, int prec, Codeboo
 cudaError_t launch_assign_fp32(const float *X, long long n, int D, int k,
                                const CodebookPrep &p, uint8_t *labels, FlagList fl,
                                cudaStream_t s);
+// A second pass over pixels that another contraction left ambiguous runs only where that one's
+// count exceeds a limit; its flag list then replaces the first one's (same entries, own counter).
+struct SecondPass {
+    const unsigned int *first;    // the first pass's counter (null: not a second pass)
+    const unsigned int *count;    // the second pass's counter
+    unsigned int limit;
+};
 cudaError_t launch_assign_bf16(const float *X, long long n, int D, int k,
                                const CodebookPrep &p, uint8_t *labels, FlagList fl,
-                               cudaStream_t s);
+                               cudaStream_t s, SecondPass second = {});
 // FP8 e4m3 contraction (quantisation of the features into f8, then tcgen05 kind::f8f6f4).
 bool fp8_supported(int D, int k);
 cudaError_t launch_assign_fp8(const float *X, long long n, int D, int k, const CodebookPrep &p, Fp8Feat f8,
@@ -71,7 +80,8 @@ cudaError_t launch_assign_fp8(const float *X, long long n, int D, int k, const C
 // Several codebooks in one contraction: p holds krows prepared rows (the segments' columns,
 // padding rows included); the sum of the segments' ncol is at most 256.
 cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const CodebookPrep &p, int krows,
-                                   const TcSeg *seg, int nseg, int sf, int pf, cudaStream_t s);
+                                   const TcSeg *seg, int nseg, int sf, int pf, cudaStream_t s,
+                                   SecondPass second = {});
 // Several groups of codebooks against one tile of features read once (the tile's BF16 operand
 // stays in tensor memory while every group's centroids stream past): p holds ngroup * gcols
 // prepared rows, group g at rows g * gcols; seg[] lists every group's segments with absolute
@@ -82,8 +92,8 @@ cudaError_t launch_assign_bf16_stat(const float *X, long long n, int D, const Co
 // Largest number of groups of gcols columns one stationary launch holds (shared memory).
 int stat_max_groups(int D, int gcols);
 cudaError_t launch_rescore(const float *X, long long n, int D, const float *C, int k,
-                           uint8_t *labels, FlagList fl, cudaStream_t s);
-cudaError_t launch_finish_stats(FlagList fl, vqnnf_assign_stats *out, cudaStream_t s);
+                           uint8_t *labels, FlagList fl, cudaStream_t s, SecondPass second = {});
+cudaError_t launch_finish_stats(FlagList fl, bool fp8, vqnnf_assign_stats *out, cudaStream_t s);
 
 // Launch with programmatic stream serialization: the kernel's blocks may be scheduled before the
 // preceding kernel of the stream finishes; every kernel launched this way calls ptx::pdl_enter()
