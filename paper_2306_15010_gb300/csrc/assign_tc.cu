@@ -1141,6 +1141,21 @@ size_t tc_smem_bytes(int npad, int D, int sb, int sf, int ncols = 0, int nsegcap
 
 }  // namespace
 
+cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int rows)
+{
+    const cudaError_t e = get_encode();
+    if (e != cudaSuccess) return e;
+    const cuuint64_t es = u16 ? 2 : 4;
+    const cuuint64_t dims[3] = {(cuuint64_t)P, (cuuint64_t)k, (cuuint64_t)rows};
+    const cuuint64_t strides[2] = {(cuuint64_t)P * es, (cuuint64_t)P * k * es};
+    const cuuint32_t box[3] = {(cuuint32_t)(128 / es), 32, 1};
+    const cuuint32_t step[3] = {1, 1, 1};
+    const CUresult r = g_encode(m, u16 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, S, dims, strides,
+                                box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const CodebookPrep &p, int krows,
                                    const TcSeg *seg, int nseg, int sf_req, int pf, cudaStream_t s, SecondPass second)
 {

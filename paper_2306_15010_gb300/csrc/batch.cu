@@ -111,12 +111,8 @@ BatchWs carve_batch(WsCursor &c, const vqnnf_image *q, int nq, const vqnnf_batch
 {
     BatchWs w;
     long long n_max = 0, l_max = 0, hw_max = 0;
-    int k_max = 1, H_max = 1, W_max = 1;
-    for (int i = 0; i < nq; ++i) {
-        n_max = std::max(n_max, (long long)q[i].H * q[i].W);
-        H_max = std::max(H_max, (int)q[i].H);
-        W_max = std::max(W_max, (int)q[i].W);
-    }
+    int k_max = 1;
+    for (int i = 0; i < nq; ++i) n_max = std::max(n_max, (long long)q[i].H * q[i].W);
     for (int j = 0; j < nt; ++j) {
         l_max = std::max(l_max, (long long)t[j].h * t[j].w);
         k_max = std::max(k_max, (int)t[j].k);
@@ -166,13 +162,14 @@ BatchWs carve_batch(WsCursor &c, const vqnnf_image *q, int nq, const vqnnf_batch
     w.sprep.v = c.take<float>(srows);
     w.sprep.b = c.take<float>(srows);
     for (int l = 0; l < kLanes; ++l) w.fit[l] = carve_fit(c, l_max, D, k_max);
-    // the largest integral-image layout over the templates (its size depends on the template)
+    // the largest integral-image layout over the pairs (small images take more bands)
     size_t sbytes = 0;
-    for (int j = 0; j < nt; ++j) {
-        WsCursor z{nullptr, 0};
-        carve_score(z, H_max, W_max, k_max, t[j].h, t[j].w);
-        sbytes = std::max(sbytes, z.off);
-    }
+    for (int i = 0; i < nq; ++i)
+        for (int j = 0; j < nt; ++j) {
+            WsCursor z{nullptr, 0};
+            carve_score(z, q[i].H, q[i].W, t[j].k, t[j].h, t[j].w);
+            sbytes = std::max(sbytes, z.off);
+        }
     for (int l = 0; l < kLanes; ++l) {
         w.score_base[l] = c.take<char>(sbytes);
         w.heat_scratch[l] = c.take<float>((size_t)hw_max);

@@ -12,7 +12,7 @@
 // 65,536 pixels (template area <= 65,535) -- the four-corner sum taken mod 2^16 is then the
 // exact count -- else uint32_t.
 //
-// Build, in bands of BH rows so that every warp sweeps few rows:
+// Build, in bands of up to 64 rows so that every warp sweeps few rows:
 //   (1) row carries: per row, the count of every cluster left of every 64-column strip;
 //   (2) band sums: per (band, strip), the column sums of the row prefixes (exact int32) =
 //       the band's carries plus the prefix along x of the band's per-column label counts;
@@ -41,7 +41,6 @@ namespace {
 __device__ int g_score_error = 0;
 
 constexpr int SW = 64;     // columns per strip (two per lane)
-constexpr int BH = 64;     // rows per band
 
 // carry[(y * nS + s) * k + j] = #{x' < 64 s : label(y, x') = j}
 __global__ void row_carry_kernel(const uint8_t *__restrict__ lab, int W, int k, int nS,
@@ -72,7 +71,7 @@ __global__ void row_carry_kernel(const uint8_t *__restrict__ lab, int W, int k, 
 // columns x = sum over the band's rows y of #{x' < x : label(y, x') = j}
 //          = sum_y carry(y, strip, j) + #{(y, x') : y in band, strip start <= x' < x, label = j}.
 __global__ void __launch_bounds__(256) band_sum_kernel(const uint8_t *__restrict__ lab, int H, int W,
-                                                       int k, int P, int nS, const int *__restrict__ carry,
+                                                       int k, int P, int nS, int BH, const int *__restrict__ carry,
                                                        int *__restrict__ bandsum)
 {
     ptx::pdl_enter();
@@ -130,50 +129,51 @@ __global__ void __launch_bounds__(256) band_sum_kernel(const uint8_t *__restrict
 // band's running S values of the strip's 64 columns in registers.  Per row the strip's labels
 // are staged in shared memory (two bytes per lane, double-buffered) and read back whole by
 // every lane; the lane walks the 64 columns once, adding its row prefix (the carry plus one
-// for every earlier column labelled j) to each column's value.  The finished row of its plane
-// goes to a padded shared-memory row (conflict-free 16-byte stores) and from there to global
-// memory as one bulk copy, double-buffered: stores of 32 lanes to 32 different planes would
-// otherwise each touch a different line.  Columns past the image carry a label byte that no
-// lane of the warp owns, so they repeat the value of column W.
+// for every earlier column labelled j) to each column's value.  The finished rows of the 32
+// planes go to a shared-memory tile (128-byte rows, 16-byte chunks swizzled as the copy expects, so
+// the lanes' stores do not conflict) and from there to global memory in one tensor copy, which
+// leaves out the planes past k.  On a 2048 x 2048 image, k = 128 (1.1 GB) the whole table takes
+// 0.29 ms; with a copy of its own for each lane's 128 bytes, 0.35 ms (4.2 TB/s in this pass: the
+// copies' issue, not the bytes).  Columns past
+// the image carry a label byte that no lane of the warp owns, so they repeat the value of column W.
+constexpr int kSatWarps = 4;                                   // warps per block
+constexpr int kSatBuf = 2;                                     // staged rows of a warp
 template <typename T>
-struct SatSweep {
-    static constexpr int warps = sizeof(T) == 2 ? 4 : 2;        // warps per block
-    static constexpr int pitch = SW * (int)sizeof(T) + 16;       // staged row bytes (padded)
+struct SatTile {
+    static constexpr int tiles = SW * (int)sizeof(T) / 128;    // 128-byte rows per plane and image row
+    static constexpr int bytes = tiles * 32 * 128;
+    static constexpr int smem = kSatWarps * (kSatBuf * bytes + 2 * SW) + 1024;
 };
 
+// 16-byte chunk g of the strip's row, as T
 template <typename T>
-__device__ __forceinline__ void pack_row(uint8_t *dst, const int (&acc)[SW]);
+__device__ __forceinline__ uint4 pack_chunk(const int (&acc)[SW], int g);
 template <>
-__device__ __forceinline__ void pack_row<uint16_t>(uint8_t *dst, const int (&acc)[SW])
+__device__ __forceinline__ uint4 pack_chunk<uint16_t>(const int (&acc)[SW], int g)
 {
-#pragma unroll
-    for (int g = 0; g < SW / 8; ++g)
-        reinterpret_cast<uint4 *>(dst)[g] = make_uint4(__byte_perm(acc[8 * g], acc[8 * g + 1], 0x5410),
-                                                       __byte_perm(acc[8 * g + 2], acc[8 * g + 3], 0x5410),
-                                                       __byte_perm(acc[8 * g + 4], acc[8 * g + 5], 0x5410),
-                                                       __byte_perm(acc[8 * g + 6], acc[8 * g + 7], 0x5410));
+    return make_uint4(__byte_perm(acc[8 * g], acc[8 * g + 1], 0x5410), __byte_perm(acc[8 * g + 2], acc[8 * g + 3], 0x5410),
+                      __byte_perm(acc[8 * g + 4], acc[8 * g + 5], 0x5410), __byte_perm(acc[8 * g + 6], acc[8 * g + 7], 0x5410));
 }
 template <>
-__device__ __forceinline__ void pack_row<uint32_t>(uint8_t *dst, const int (&acc)[SW])
+__device__ __forceinline__ uint4 pack_chunk<uint32_t>(const int (&acc)[SW], int g)
 {
-#pragma unroll
-    for (int g = 0; g < SW / 4; ++g)
-        reinterpret_cast<uint4 *>(dst)[g] = make_uint4((uint32_t)acc[4 * g], (uint32_t)acc[4 * g + 1],
-                                                       (uint32_t)acc[4 * g + 2], (uint32_t)acc[4 * g + 3]);
+    return make_uint4((uint32_t)acc[4 * g], (uint32_t)acc[4 * g + 1], (uint32_t)acc[4 * g + 2], (uint32_t)acc[4 * g + 3]);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
-    const uint8_t *__restrict__ lab, int H, int W, int k, int P, int nS, int nB, const int *__restrict__ carry,
-    const int *__restrict__ bandsum, T *__restrict__ S, T *__restrict__ coarse)
+__global__ void __launch_bounds__(32 * kSatWarps, 4) sat_write_kernel(
+    const __grid_constant__ CUtensorMap map, const uint8_t *__restrict__ lab, int H, int W, int k, int P, int nS, int nB,
+    int BH, const int *__restrict__ carry, const int *__restrict__ bandsum, T *__restrict__ coarse)
 {
     ptx::pdl_enter();
-    constexpr int NW = SatSweep<T>::warps, PITCH = SatSweep<T>::pitch;
-    __shared__ __align__(16) uint8_t srow[NW][2][SW];
-    __shared__ __align__(16) uint8_t sout[NW][2][32][PITCH];
+    using L = SatTile<T>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    uint8_t *sout = base + wi * kSatBuf * L::bytes;
+    uint8_t *srow = base + kSatWarps * kSatBuf * L::bytes + wi * 2 * SW;
     const int ncg = (k + 31) >> 5;
-    const long long gw = (long long)blockIdx.x * NW + wi;
+    const long long gw = (long long)blockIdx.x * kSatWarps + wi;
     if (gw >= (long long)nB * nS * ncg) return;              // uniform over the warp
     const int s = (int)(gw % nS);                            // adjacent warps: adjacent strips
     const int cg = (int)((gw / nS) % ncg);
@@ -182,8 +182,6 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
     const bool jin = j < k;
     const int jc = jin ? j : k - 1;                          // clamped (every address in bounds)
     const int x0 = s * SW;
-    const int ncolv = min(SW, P - x0);                       // S columns of the strip: a multiple of 8
-    const uint32_t row_bytes = (uint32_t)(ncolv * (int)sizeof(T));   // a multiple of 16
     const int kp = sat_coarse_pitch(k);
     const int y0 = b * BH, y1 = min(H, y0 + BH);
     const uint32_t fill = (uint32_t)(((cg + 1) * 32) & 0xFF);   // outside [32 cg, 32 cg + 31]
@@ -194,32 +192,43 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
         const int *src = bandsum + ((size_t)b * k + jc) * P + x0;
 #pragma unroll
         for (int g = 0; g < SW / 4; ++g) {
-            int4 v = make_int4(0, 0, 0, 0);
-            if (4 * g < ncolv) v = *reinterpret_cast<const int4 *>(src + 4 * g);
+            const int4 v = *reinterpret_cast<const int4 *>(src + 4 * g);
             acc[4 * g] = v.x;
             acc[4 * g + 1] = v.y;
             acc[4 * g + 2] = v.z;
             acc[4 * g + 3] = v.w;
         }
     }
-    // row yrow of this lane's plane, through staging buffer bsel; a buffer is rewritten only
-    // once the copy committed two rows earlier has read it
+    // row yrow of the 32 planes, through staging buffer bsel; a buffer is rewritten only once the
+    // copy committed kSatBuf rows earlier (by lane 0) has read it
     auto emit = [&](int yrow, int bsel) {
-        if (!jin) return;
-        uint8_t *st = &sout[wi][bsel][lane][0];
-        ptx::bulk_wait_read<1>();
-        pack_row<T>(st, acc);
+        uint8_t *st = sout + bsel * L::bytes;
+        if (lane == 0) ptx::bulk_wait_read<kSatBuf - 1>();
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < L::tiles; ++t)
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                *reinterpret_cast<uint4 *>(st + t * 4096 + lane * 128 + ((g ^ (lane & 7)) << 4)) = pack_chunk<T>(acc, 8 * t + g);
         ptx::fence_proxy_async();
-        ptx::bulk_s2g(S + ((size_t)yrow * k + j) * P + x0, st, row_bytes);
-        ptx::bulk_commit();
-        if (yrow % kCoarseY == 0 || yrow == H) {              // the coarse samples of this row
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+            for (int t = 0; t < L::tiles; ++t) ptx::tma_store_3d(&map, st + t * 4096, x0 + t * (SW / L::tiles), cg * 32, yrow);
+            ptx::bulk_commit();
+        }
+        if (jin && (yrow % kCoarseY == 0 || yrow == H)) {     // the coarse samples of this row
             T *c = coarse + ((size_t)((yrow + kCoarseY - 1) / kCoarseY) * sat_coarse_cols(W) + x0 / kCoarseX) * kp + j;
 #pragma unroll
             for (int u = 0; u < SW / kCoarseX; ++u) c[(size_t)u * kp] = (T)acc[u * kCoarseX];
             if (s == nS - 1) c[(size_t)(SW / kCoarseX) * kp] = (T)acc[SW - 1];
         }
     };
-    if (b == 0) emit(0, 1);                                   // row 0 of S (all zero)
+    int bsel = 0;
+    if (b == 0) {                                             // row 0 of S (all zero)
+        emit(0, bsel);
+        bsel ^= 1;
+    }
     // labels and carry of the next row are loaded one row ahead; lane l stages columns
     // x0 + 2l and x0 + 2l + 1
     const int xa = x0 + 2 * lane;
@@ -232,7 +241,7 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
         c_n = carry[((size_t)y0 * nS + s) * k + jc];
     }
     for (int y = y0; y < y1; ++y) {
-        uint8_t *buf = srow[wi][y & 1];
+        uint8_t *buf = srow + (y & 1) * SW;
         buf[2 * lane] = (uint8_t)la_n;
         buf[2 * lane + 1] = (uint8_t)lb_n;
         int rp = c_n;
@@ -261,9 +270,10 @@ __global__ void __launch_bounds__(32 * SatSweep<T>::warps, 4) sat_write_kernel(
                 rp += (d & (0xFFu << (8 * u))) == 0u ? 1 : 0;
             }
         }
-        emit(y + 1, y & 1);
+        emit(y + 1, bsel);
+        bsel ^= 1;
     }
-    ptx::bulk_wait_read<0>();                                 // staging rows read before the block exits
+    if (lane == 0) ptx::bulk_wait_read<0>();                  // staging rows read before the block exits
 }
 
 // Exclusive prefix of the band sums over bands, per (cluster, column), in place.
@@ -554,7 +564,7 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
 {
     const int nS = sat_strips(W);
     const int P = sat_pitch(W);
-    const int nB = sat_bands(H);
+    const int BH = sat_band_rows(H, W, k), nB = sat_bands(H, W, k);
     const size_t hsmem = sizeof(int) * (size_t)nS * k;
     cudaError_t e = cudaFuncSetAttribute(row_carry_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsmem);
@@ -567,7 +577,7 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
     e = cudaFuncSetAttribute(band_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem);
     if (e != cudaSuccess) return e;
     {
-        const cudaError_t le_ = launch_pdl(band_sum_kernel, dim3(dim3(nS, nB)), dim3(256), csmem, s, lab, H, W, k, P, nS, carry, bandsum);
+        const cudaError_t le_ = launch_pdl(band_sum_kernel, dim3(dim3(nS, nB)), dim3(256), csmem, s, lab, H, W, k, P, nS, BH, carry, bandsum);
         if (le_ != cudaSuccess) return le_;
     }
     const long long kP = (long long)k * P;
@@ -576,12 +586,15 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
         if (le_ != cudaSuccess) return le_;
     }
     const long long nwarps = (long long)nB * nS * ((k + 31) / 32);
-    constexpr int NW = SatSweep<T>::warps;
-    const unsigned blocks = (unsigned)((nwarps + NW - 1) / NW);
-    {
-        const cudaError_t le_ = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * NW), 0, s, lab, H, W, k, P, nS, nB, carry, bandsum, S, coarse);
-        if (le_ != cudaSuccess) return le_;
-    }
+    const unsigned blocks = (unsigned)((nwarps + kSatWarps - 1) / kSatWarps);
+    CUtensorMap map;
+    e = make_sat_map(&map, S, sizeof(T) == 2, P, k, H + 1);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(sat_write_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SatTile<T>::smem);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * kSatWarps), SatTile<T>::smem, s, map, lab, H, W, k, P, nS, nB,
+                   BH, carry, bandsum, coarse);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -629,7 +642,20 @@ size_t score_smem_bytes_for(size_t elem, const BankSpec &bs, const GridSpec &gs,
 bool sat_is_u16(int th, int tw) { return (long long)th * tw <= 65535; }
 int sat_pitch(int W) { return (W + 1 + 63) / 64 * 64; }
 int sat_strips(int W) { return (W + 1 + SW - 1) / SW; }
-int sat_bands(int H) { return (H + BH - 1) / BH; }
+// Rows of a band: 64, halved (down to 8) while the write pass has fewer than eight warps per SM -- it
+// sweeps a band's rows one after another, and so few warps leave it waiting for memory (256 x 256,
+// k = 16: 20 warps of 64 rows took 62 us, the table 75 us; 25 us in all with bands of 8 rows).
+int sat_band_rows(int H, int W, int k)
+{
+    int bh = 64;
+    while (bh > 8 && (long long)((H + bh - 1) / bh) * sat_strips(W) * ((k + 31) / 32) < 1216) bh /= 2;
+    return bh;
+}
+int sat_bands(int H, int W, int k)
+{
+    const int bh = sat_band_rows(H, W, k);
+    return (H + bh - 1) / bh;
+}
 int score_ncol(int tw) { return (TXW + tw + 7) / 8 * 8; }
 size_t sat_slack_elems(int tw) { return (size_t)score_ncol(tw) + 64; }
 

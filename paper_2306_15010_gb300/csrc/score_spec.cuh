@@ -1,6 +1,7 @@
 // Filter-bank descriptions passed to the score kernels by value (kernel parameters).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -75,7 +76,11 @@ __host__ __device__ inline int sat_coarse_rows(int H) { return (H + kCoarseY - 1
 bool sat_is_u16(int th, int tw);
 int sat_pitch(int W);
 int sat_strips(int W);
-int sat_bands(int H);
+int sat_band_rows(int H, int W, int k);
+int sat_bands(int H, int W, int k);
+// Tensor map of the integral image for the write pass: 32 planes x 128 bytes of one row (assign_tc.cu,
+// beside the other maps).
+cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int rows);
 int score_ncol(int tw);
 bool score_grid_fits(int ncol);   // the grid kernel stages at most TXW + 256 columns
 size_t sat_slack_elems(int tw);
