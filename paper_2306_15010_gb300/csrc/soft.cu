@@ -22,6 +22,7 @@
 #include <cfloat>
 
 #include "common.cuh"
+#include "ptx.cuh"
 #include "soft_spec.cuh"
 
 namespace vqnnf {
@@ -268,6 +269,106 @@ __global__ void col_box_kernel(const float *__restrict__ RW, int H, int W, int h
     for (int y = y0 + 1; y < ye; ++y) {
         s += src[(size_t)(y + h - 1) * W] - src[(size_t)(y - 1) * W];
         BX[(plane * H + y) * W + x] = s;
+    }
+}
+
+// Asynchronous copies of 4 and 16 (past L1) bytes into shared memory, or as many zeros.
+__device__ __forceinline__ void cp4_or_zero(float *dst, const float *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp16_or_zero(float *dst, const float *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// All of a plane's box sums at once: a block takes BXT x BYT outputs, stages the pixels under them,
+// forms the row sums of both widths (the larger is one more, if there are two) from there into
+// shared memory, and from these the column sums of both heights, in the order of row_box_kernel and
+// col_box_kernel (segments of SEG outputs from multiples of SEG: the same values).  The two widths,
+// and the two heights, share their loads: a step of the sliding sums is one new value and one old.
+//
+// Bound by the writes of the box sums (one map per size class; the pixels are read about once from
+// HBM and (1 + w / BXT)(1 + h / BYT) times from L2) and by shared memory (some five accesses an output).
+// 8 x 512 x 512, k = 64, cells of 21 or 22: 0.75 ms; 1.88 ms as a row pass per width and a column pass
+// per class and item, 1.21 ms with loads through registers (too few in flight).
+constexpr int BXT = 64, BYT = 32;
+struct BoxSpec {
+    int wlo, hlo;                  // smaller width and height
+    int cls[2][2];                 // size class of [width][height], smaller first
+};
+__host__ __device__ constexpr int box_rows(int hlo) { return BYT + hlo; }
+__host__ __device__ constexpr int box_cols(int wlo) { return (BXT + wlo) | 1; }   // odd: lanes on rows do not conflict
+size_t box_smem(int nw, int wlo, int hlo) { return sizeof(float) * box_rows(hlo) * (size_t)(box_cols(wlo) + nw * (BXT + 1)); }
+
+template <int NW, int NH>
+__global__ void __launch_bounds__(256) box_kernel(const float *__restrict__ P, int H, int W, int k, int ns, BoxSpec bs,
+                                                  float *__restrict__ BX)
+{
+    extern __shared__ float bsm[];
+    const int wlo = bs.wlo, hlo = bs.hlo, nr = box_rows(hlo), pc = box_cols(wlo);
+    float *ps = bsm, *rs = bsm + nr * pc;                     // pixels; row sums [NW][nr][BXT + 1]
+    const int x0 = blockIdx.x * BXT, y0 = blockIdx.y * BYT;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const size_t plane = (size_t)H * W;
+    const float *src = P + blockIdx.z * plane;
+    for (int r = warp; r < nr; r += 8) {
+        const float *row = src + (size_t)min(y0 + r, H - 1) * W;
+        for (int c = lane; c < BXT + wlo; c += 32)
+            cp4_or_zero(ps + r * pc + c, row + min(x0 + c, W - 1), y0 + r < H && x0 + c < W);
+    }
+    cp_commit();
+    cp_wait<0>();
+    __syncthreads();
+    for (int e = t; e < nr * (BXT / SEG); e += 256) {
+        const int sg = e / nr, r = e - sg * nr;
+        const float *p = ps + r * pc + sg * SEG;
+        float *o = rs + r * (BXT + 1) + sg * SEG;
+        float lo = 0.f;
+        for (int dx = 0; dx < wlo; ++dx) lo += p[dx];
+        float nxt = p[wlo], hi = lo + nxt;
+        o[0] = lo;
+        if (NW == 2) o[nr * (BXT + 1)] = hi;
+#pragma unroll
+        for (int i = 1; i < SEG; ++i) {
+            const float cur = nxt, old = p[i - 1];
+            if (NW == 2 || i < SEG - 1) nxt = p[i + wlo];
+            lo += cur - old;
+            o[i] = lo;
+            if (NW == 2) {
+                hi += nxt - old;
+                o[nr * (BXT + 1) + i] = hi;
+            }
+        }
+    }
+    __syncthreads();
+    const int x = t & (BXT - 1), sg = t / BXT, gx = x0 + x, gy = y0 + sg * SEG;   // BYT / SEG segments
+    const int b = blockIdx.z / k, j = blockIdx.z - b * k;
+#pragma unroll
+    for (int iw = 0; iw < NW; ++iw) {
+        if (gx > W - (wlo + iw)) continue;
+        const float *q = rs + (iw * nr + sg * SEG) * (BXT + 1) + x;
+        float *out[NH];
+#pragma unroll
+        for (int ih = 0; ih < NH; ++ih)
+            out[ih] = BX + ((size_t)(b * ns + bs.cls[iw][ih]) * k + j) * plane + (size_t)gy * W + gx;
+        float lo = 0.f;
+        for (int dy = 0; dy < hlo; ++dy) lo += q[dy * (BXT + 1)];
+        float nxt = q[hlo * (BXT + 1)], hi = lo + nxt;
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) {
+            if (i > 0) {
+                const float cur = nxt, old = q[(i - 1) * (BXT + 1)];
+                nxt = q[(i + hlo) * (BXT + 1)];
+                lo += cur - old;
+                hi += nxt - old;
+            }
+            if (gy + i <= H - hlo) out[0][(size_t)i * W] = lo;
+            if (NH == 2 && gy + i <= H - hlo - 1) out[NH - 1][(size_t)i * W] = hi;
+        }
     }
 }
 
@@ -572,6 +673,68 @@ struct AdjCols {
     int ns;
     int h[4];
 };
+// A block takes BXT x BYT outputs and stages the rows above them that count (rows outside
+// [0, H - h_s] as zeros), the next class's while the current one is summed; the sums are those of
+// adj_col_kernel in the same order.  Bound by the reads (each row once from HBM, 1 + h / BYT times from
+// L2).  Rows that start on 16 bytes are copied in chunks of that.
+// 8 x 512 x 512, k = 64: 0.55 ms; 1.20 ms straight from global memory (adj_col_kernel), 1.01 ms
+// staged through registers class by class.
+size_t adj_smem(int hmax) { return sizeof(float) * 2 * (BYT + hmax - 1) * (size_t)BXT; }
+__global__ void __launch_bounds__(256) adj_tile_kernel(const float *__restrict__ R2, long long cls_stride, int H, int W,
+                                                       const __grid_constant__ AdjCols ac, int hmax, bool vec,
+                                                       float *__restrict__ Gp)
+{
+    extern __shared__ __align__(16) float bsm[];
+    const int x0 = blockIdx.x * BXT, y0 = blockIdx.y * BYT;
+    const int t = threadIdx.x, x = t & (BXT - 1), sg = t / BXT, gx = x0 + x, gy = y0 + sg * SEG;
+    const long long plane = blockIdx.z;
+    const int buf = (BYT + hmax - 1) * BXT;
+    auto stage = [&](int is) {
+        const int h = ac.h[is], ym = H - h, nr = BYT + h - 1;
+        const float *src = R2 + is * cls_stride + plane * H * W;
+        float *dst = bsm + (is & 1) * buf;
+        if (vec) {
+            const int c = 4 * (t & 15), cx = min(x0 + c, W - 4);
+            for (int r = t >> 4; r < nr; r += 16) {
+                const int y = y0 - h + 1 + r;
+                cp16_or_zero(dst + r * BXT + c, src + (size_t)min(max(y, 0), ym) * W + cx, y >= 0 && y <= ym && x0 + c < W);
+            }
+        } else {
+            for (int r = sg; r < nr; r += 256 / BXT) {
+                const int y = y0 - h + 1 + r;
+                cp4_or_zero(dst + r * BXT + x, src + (size_t)min(max(y, 0), ym) * W + min(gx, W - 1), y >= 0 && y <= ym && gx < W);
+            }
+        }
+    };
+    stage(0);
+    cp_commit();
+    float out[SEG];
+#pragma unroll
+    for (int i = 0; i < SEG; ++i) out[i] = 0.f;
+    for (int is = 0; is < ac.ns; ++is) {
+        if (is + 1 < ac.ns) stage(is + 1);
+        cp_commit();
+        cp_wait<1>();
+        __syncthreads();
+        const int h = ac.h[is];
+        const float *q = bsm + (is & 1) * buf + sg * SEG * BXT + x;
+        float s = 0.f;
+#pragma unroll 4
+        for (int r = 0; r < h; ++r) s += q[r * BXT];
+        out[0] += s;
+#pragma unroll
+        for (int i = 1; i < SEG; ++i) {
+            s += q[(h - 1 + i) * BXT];
+            s -= q[(i - 1) * BXT];
+            out[i] += s;
+        }
+        __syncthreads();                                      // the buffer may be refilled
+    }
+    if (gx >= W) return;
+#pragma unroll
+    for (int i = 0; i < SEG; ++i)
+        if (gy + i < H) Gp[(plane * H + gy + i) * W + gx] = out[i];
+}
 __global__ void adj_col_kernel(const float *__restrict__ R2, long long cls_stride, int H, int W, AdjCols ac,
                                float *__restrict__ Gp)
 {
@@ -847,6 +1010,27 @@ cudaError_t launch_soft_back(const float *X, long long n, long long npi, int D, 
     return launch_soft_back_ki<8>(X, n, npi, D, C, k, tau, P, Gp, A, dX, s);
 }
 
+constexpr size_t kTileSmem = 100 * 1024;
+BoxSpec box_spec(const SoftGrid &sg)
+{
+    BoxSpec bs = {};
+    const int wl = sg.nw == 2 && sg.wid[1] < sg.wid[0], hl = sg.nh == 2 && sg.hgt[1] < sg.hgt[0];   // index of the smaller
+    bs.wlo = sg.wid[wl];
+    bs.hlo = sg.hgt[hl];
+    for (int s = 0; s < sg.ns; ++s) bs.cls[sg.size_w[s] != wl][sg.size_h[s] != hl] = s;
+    return bs;
+}
+
+template <int NW, int NH>
+cudaError_t launch_box(SoftWs &w, int B, int H, int W, int k, const SoftGrid &sg, const BoxSpec &bs, size_t smem, cudaStream_t s)
+{
+    const cudaError_t e = cudaFuncSetAttribute(box_kernel<NW, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    box_kernel<NW, NH><<<dim3((W - bs.wlo + BXT) / BXT, (H - bs.hlo + BYT) / BYT, (unsigned)(B * k)), 256, smem, s>>>(
+        w.P, H, W, k, sg.ns, bs, w.BX);
+    return cudaGetLastError();
+}
+
 template <int MC, int J>
 cudaError_t launch_gather_j(const SoftWs &w, const float *dheat, const float *wf, int B, int H, int W, int k, int HO,
                             int WO, const SoftGrid &sg, int is, cudaStream_t s)
@@ -949,7 +1133,17 @@ cudaError_t soft_forward(const float *Qf, int B, int H, int W, const float *Tf, 
     e = launch_soft_p(Tf, nt, nt, D, C, k, tau, w.Pt, s);
     if (e != cudaSuccess) return e;
     const long long planes = (long long)B * k;
-    for (int iw = 0; iw < sg.nw; ++iw) {
+    const BoxSpec bx = box_spec(sg);
+    const size_t bsm = box_smem(sg.nw, bx.wlo, bx.hlo);
+    // Cells up to about 60 a side: two blocks of the tile's shared memory fit an SM.  There (cells of
+    // 58 and 59, a training step of 2 x 512 x 512, k = 64) both ways take 1.30 ms.
+    const bool fused = bsm <= kTileSmem;
+    if (fused) {
+        e = sg.nw == 1 ? (sg.nh == 1 ? launch_box<1, 1>(w, B, H, W, k, sg, bx, bsm, s) : launch_box<1, 2>(w, B, H, W, k, sg, bx, bsm, s))
+                       : (sg.nh == 1 ? launch_box<2, 1>(w, B, H, W, k, sg, bx, bsm, s) : launch_box<2, 2>(w, B, H, W, k, sg, bx, bsm, s));
+        if (e != cudaSuccess) return e;
+    }
+    for (int iw = 0; iw < sg.nw && !fused; ++iw) {
         const int wd = sg.wid[iw];
         const size_t rs = row_box_smem(wd);                   // up to ~56 KB (W <= 12288)
         e = cudaFuncSetAttribute(row_box_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
@@ -957,7 +1151,7 @@ cudaError_t soft_forward(const float *Qf, int B, int H, int W, const float *Tf, 
         dim3 g((unsigned)(planes * H), (W - wd + RBX) / RBX);
         row_box_kernel<<<g, 128, rs, s>>>(w.P, W, wd, w.RW + (size_t)iw * planes * H * W);
     }
-    for (int is = 0; is < sg.ns; ++is) {
+    for (int is = 0; is < sg.ns && !fused; ++is) {
         const int iw = sg.size_w[is];
         for (int b = 0; b < B; ++b) {
             dim3 g((W + 127) / 128, (H + SEG - 1) / SEG, k);
@@ -998,8 +1192,18 @@ cudaError_t soft_backward(const float *Qf, int B, int H, int W, const float *Tf,
         if (e != cudaSuccess) return e;
         ac.h[is] = h;
     }
-    dim3 g3((W + 127) / 128, (H + SEG - 1) / SEG, (unsigned)planes);
-    adj_col_kernel<<<g3, 128, 0, s>>>(w.R2, planes * H * W, H, W, ac, w.G);
+    int hmax = 0;
+    for (int is = 0; is < sg.ns; ++is) hmax = ac.h[is] > hmax ? ac.h[is] : hmax;
+    const size_t csm = adj_smem(hmax);
+    if (csm <= kTileSmem) {
+        e = cudaFuncSetAttribute(adj_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+        if (e != cudaSuccess) return e;
+        adj_tile_kernel<<<dim3((W + BXT - 1) / BXT, (H + BYT - 1) / BYT, (unsigned)planes), 256, csm, s>>>(
+            w.R2, planes * H * W, H, W, ac, hmax, W % 4 == 0, w.G);
+    } else {
+        dim3 g3((W + 127) / 128, (H + SEG - 1) / SEG, (unsigned)planes);
+        adj_col_kernel<<<g3, 128, 0, s>>>(w.R2, planes * H * W, H, W, ac, w.G);
+    }
     const size_t kDk = (size_t)k * D + k;
     if (soft_tc_supported(D, k)) {                            // tensor-core contractions
         int nqs = 0, nts = 0;
