@@ -461,8 +461,8 @@ __global__ void soft_dw_kernel(const float *__restrict__ dheat, const float *__r
 // 0, and everything else on packed pairs of planes, each component rounded as the scalar operation
 // (the product with 1, 0 or -1 is exact).  A weight that is not finite takes selects instead (0 times
 // it would not be 0).
-// 8 x 512 x 512 pixels, k = 64, cells of 21 or 22: 2.41 ms for the four classes (0.55 ms for the one
-// of a single cell), 2.91 ms with selects, thresholds in shared memory and room for four cells always.
+// 8 x 512 x 512 pixels, k = 64, cells of 21 or 22: 2.19 ms for the four classes (0.47 ms for the one
+// of a single cell), 2.39 ms with two blocks an SM for all of them, 2.91 ms with selects, thresholds in shared memory and room for four cells always.
 constexpr int GR = 2;              // rows per block of the gradient gather
 constexpr int SG = 32;             // outputs per thread segment of its row pass
 __host__ __device__ constexpr int gather_pitch(int W) { return W + W / 32 + 1; }   // skewed row
@@ -473,7 +473,7 @@ __device__ __forceinline__ float above(float a, float b)   // a > b ? 1 : 0
     return r;
 }
 template <int MC, int J>           // MC >= number of cells in class s; J planes per block
-__global__ void __launch_bounds__(256, MC <= 4 ? 2 : 1) soft_gather_kernel(const float *__restrict__ BX, const float *__restrict__ dheat,
+__global__ void __launch_bounds__(256, MC <= 2 ? 3 : MC <= 4 ? 2 : 1) soft_gather_kernel(const float *__restrict__ BX, const float *__restrict__ dheat,
                                                           const float *__restrict__ T, const float *__restrict__ wf,
                                                           int H, int W, int k, int HO, int WO, SoftGrid sg, int s,
                                                           float *__restrict__ R2, float *__restrict__ dT)
