@@ -168,13 +168,13 @@ struct GridTile {
     static constexpr int PER = (NCH + 31) / 32;              // per lane
     static constexpr int STAGE = NCH * 16;
 };
-// A pair to visit: slot, cluster and template count (below 2^16 where the table is 16-bit: a
-// template of at most 65,535 pixels).
+// A pair to visit: slot, cluster and template count.  Where the table is 16-bit no window's count
+// exceeds 65,535, so a larger template count (a caller's own) gives the same minimum cut to that.
 template <typename T> struct PairOf;
 template <> struct PairOf<uint16_t> {
     uint32_t v;
     PairOf() = default;
-    __device__ __forceinline__ PairOf(int q, int j, int t) : v((uint32_t)t << 16 | (uint32_t)q << 8 | (uint32_t)j) {}
+    __device__ __forceinline__ PairOf(int q, int j, int t) : v((uint32_t)min(t, 65535) << 16 | (uint32_t)q << 8 | (uint32_t)j) {}
     __device__ __forceinline__ int t() const { return (int)(v >> 16); }
     __device__ __forceinline__ int q() const { return (int)(v >> 8 & 255u); }
     __device__ __forceinline__ int j() const { return (int)(v & 255u); }
@@ -348,10 +348,7 @@ __global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 14 : 1) score_grid_t
 // tiles of 64 x 4 windows and the grids unrolled 0.67 ms (fewer warps, instruction cache).  It stays
 // the faster one on labels without any coherence (1.44 against 2.26 ms).
 constexpr int kWX = 1, kWY = 4;    // tile: 32 kWX x kWY windows
-#ifndef WNSTV
-#define WNSTV 2
-#endif
-constexpr int WNST = WNSTV;
+constexpr int WNST = 2;
 template <typename T>
 struct WTile {
     static constexpr int E = 16 / (int)sizeof(T);

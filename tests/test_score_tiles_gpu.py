@@ -89,3 +89,15 @@ def test_weighted_grid_tiles_equal_oracle(vq, H, W, th, tw, k, gauss):
     bound = 0.5 * min(f["w_f"] / f["area"] * min(abs(r[4]) for r in f["rects"]) for f in bank)
     # float32 sums of 15 terms of magnitude up to |H|: 16 roundings of 2^-24 |H| each at most
     assert np.abs(heat - ref).max() < bound + 16 * 2.0 ** -24 * np.abs(ref).max()
+
+
+def test_tiles_counts_beyond_the_table(vq):
+    """Template counts of a caller's own beyond 65,535, over a 16-bit table."""
+    H, W, th, tw, k = 160, 1100, 32, 29, 17
+    lab = _labels(H, W, k, 0.02, 3)
+    bank = synth.grid_bank(th, tw, 3, full=True)
+    tc = oracle.filter_counts(lab[5:5 + th, 3:3 + tw].astype(np.int32), k, bank)
+    tc[:, ::2] += 65537
+    heat, _ = _score(vq, lab, k, th, tw, bank, tc)
+    band, _ = _score(vq, lab[:40 + th - 1], k, th, tw, bank, tc)          # few tiles: the dense kernel
+    assert np.array_equal(band, heat[:40])
