@@ -58,9 +58,6 @@ constexpr double kU = 5.9604644775390625e-08;
 constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
 constexpr int PF = 0;              // chunks prefetched into L2 ahead of the loads (none: measured best)
 
-// Flagged pixels that an epilogue warp holds back: pixel, segment, candidate mask.
-constexpr int kPush = 32, kPushWords = 2 + kMaskWords;
-
 struct TcArgs {
     SecondPass second;
     long long n;
@@ -297,7 +294,6 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
              *nrm_empty = nrm_full + 2, *drain = nrm_empty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    uint32_t *pushbuf = tmem_slot + 4;                     // [4 epilogue warps][kPush][kPushWords]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // tensor memory: NB accumulator buffers of npad columns, then SA A-operand stages of 64
@@ -588,32 +584,6 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
         const float cnorm0 = sqrtf(mx0.x) * 1.0001f, nrm0 = mx0.x * 1.0001f;
         uint8_t *const labels0 = g.seg[0].labels;
         const FlagList fl0 = g.seg[0].fl;
-        // Flagged pixels wait in shared memory until kPush of them go out together: the flag lists'
-        // counters answer after about 2 us, which a warp used to wait for at every tile with a
-        // flagged pixel (0.2 % of the pixels made a 720 x 1280 image of D = 32, k = 128 take 218
-        // instead of 138 us).
-        uint32_t *const push = pushbuf + (warp - 18) * kPush * kPushWords;
-        int npush = 0;                                       // uniform over the warp
-        auto flush = [&]() {
-            __syncwarp();
-            const uint32_t *e = push + lane * kPushWords;
-            const bool mine = lane < npush;
-            const FlagList fl = MULTI ? segt[mine ? e[1] : 0u].fl : fl0;
-            unsigned slot = 0;
-            if (MULTI) {
-                if (mine) slot = atomicAdd(fl.count, 1u);
-            } else {
-                if (lane == 0) slot = atomicAdd(fl.count, (unsigned)npush);
-                slot = __shfl_sync(0xffffffffu, slot, 0) + (unsigned)lane;
-            }
-            if (mine && slot < (unsigned long long)g.n) {
-                fl.pix[slot] = e[0];
-#pragma unroll
-                for (int w = 0; w < kMaskWords; ++w) fl.mask[(size_t)slot * kMaskWords + w] = e[2 + w];
-            }
-            __syncwarp();
-            npush = 0;
-        };
         // One segment of this tile: prepared columns [cb, ce), whose accumulators sit at TMEM
         // column c - cshift of taddr; `release` frees the accumulator buffer after its last read.
         auto segment = [&](int sgi, uint32_t taddr, int cshift, float X, float Y, float nx, long long pix,
@@ -727,21 +697,25 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
                 mbar_arrive(&acc_empty[buf]);
             }
             uint8_t *const labels = MULTI ? segt[sgi].labels : labels0;
+            const FlagList fl = MULTI ? segt[sgi].fl : fl0;
             const int lab = (cnt == 1 ? last : amin) - cb;
             if (valid) labels[pix] = (uint8_t)lab;
             const bool flagged = valid && cnt > 1;
             const unsigned ballot = __ballot_sync(0xffffffffu, flagged);
             if (ballot) {
-                const int m = __popc(ballot);
-                if (npush + m > kPush) flush();
+                const int leader = __ffs(ballot) - 1;
+                unsigned basei = 0;
+                if (lane == leader) basei = atomicAdd(fl.count, (unsigned)__popc(ballot));
+                basei = __shfl_sync(0xffffffffu, basei, leader);
                 if (flagged) {
-                    uint32_t *e = push + (npush + __popc(ballot & ((1u << lane) - 1u))) * kPushWords;
-                    e[0] = (uint32_t)pix;
-                    e[1] = (uint32_t)sgi;
+                    const unsigned slot = basei + __popc(ballot & ((1u << lane) - 1u));
+                    if (slot < (unsigned long long)g.n) {
+                        fl.pix[slot] = (unsigned)pix;
 #pragma unroll
-                    for (int w = 0; w < kMaskWords; ++w) e[2 + w] = maskbuf[r * kMaskWords + w];
+                        for (int w = 0; w < kMaskWords; ++w)
+                            fl.mask[(size_t)slot * kMaskWords + w] = maskbuf[r * kMaskWords + w];
+                    }
                 }
-                npush += m;
             }
         };
         uint32_t tl = 0, gl = 0;
@@ -785,7 +759,6 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
                 }
             }
         }
-        if (npush) flush();
     }
 
     __syncwarp();
@@ -1163,7 +1136,6 @@ size_t tc_smem_bytes(int npad, int D, int sb, int sf, int ncols = 0, int nsegcap
     b += sizeof(uint32_t) * TM * kMaskWords;
     b += (sizeof(float4) + sizeof(TcSeg)) * nsegcap;
     b += sizeof(uint64_t) * (2 * sf + 2 * kMaxSA + 2 * kMaxSB + 8 + 1) + 16;   // barriers, TMEM slot, abort flag
-    b += sizeof(uint32_t) * 4 * kPush * kPushWords;
     return b;
 }
 
