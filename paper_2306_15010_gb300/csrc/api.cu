@@ -172,9 +172,11 @@ vqnnf_status run_assign(const float *X, long long n, int D, const float *C, int 
     // candidates each; re-scoring streams a centroid per candidate from L2.  Above an eighth of the
     // pixels the BF16 contraction, whose bound leaves 2 %, decides first: it costs one more pass over
     // the features (1024 x 1024, D = 1024, k = 128, 70 % ambiguous: 0.9 ms, re-scoring all of them
-    // 10.6 ms; an eighth of the pixels at 20 candidates re-score in 1.9 ms, at 8 in 0.8 ms).
+    // 10.6 ms; an eighth of the pixels at 20 candidates re-score in 1.9 ms, at 8 in 0.8 ms).  Where n D
+    // is below 2^21 the launch alone (7 us) costs more than re-scoring, which the chip then does in
+    // about one wave (a 16 x 19 template, D = 160: 25 us per Lloyd step without it, 33 us with it).
     SecondPass second = {};
-    if (e == cudaSuccess && prec == VQNNF_PREC_FP8) {
+    if (e == cudaSuccess && prec == VQNNF_PREC_FP8 && n * D >= (1ll << 21)) {
         CodebookPrep p = w.prep;
         p.a = w.prep.a2;
         p.v = w.prep.v2;

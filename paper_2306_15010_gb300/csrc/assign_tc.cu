@@ -259,14 +259,16 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b, float &ra, float
 // segment's bounds and bound maxima out of the tile loop.  STAT (with MULTI): several groups
 // of npad columns per tile; the tile's A stages (all nkc chunks) stay in tensor memory until
 // the last group's MMAs, and every group's centroid chunks stream through the B stages.
-template <bool MULTI, bool STAT>
+// SECOND: a second pass (SecondPass); apart, because the check takes registers that the others' epilogue
+// lacks (8 to 52 bytes of spills).
+template <bool MULTI, bool STAT, bool SECOND = false>
 __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmBhi,
                                                           const __grid_constant__ CUtensorMap tmBlo,
                                                           const __grid_constant__ TcArgs g)
 {
     ptx::pdl_enter();
-    if (g.second.first && *g.second.first <= g.second.limit) return;   // uniform over the grid
+    if (SECOND && *g.second.first <= g.second.limit) return;   // uniform over the grid
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int npad = g.npad, D = g.D, nkc = g.nkc, SB = g.sb, SF = g.sf, NB = g.nb, SA = g.sa;
@@ -1159,7 +1161,8 @@ cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int ro
 cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const CodebookPrep &p, int krows,
                                    const TcSeg *seg, int nseg, int sf_req, int pf, cudaStream_t s, SecondPass second)
 {
-    if (D % 16 != 0 || nseg < 1 || nseg > kMaxSeg || krows < 1 || n < 1) return cudaErrorNotSupported;
+    if (D % 16 != 0 || nseg < 1 || nseg > kMaxSeg || krows < 1 || n < 1 || (second.first && nseg > 1))
+        return cudaErrorNotSupported;
     int npad = 0;
     for (int q = 0; q < nseg; ++q) {
         if (seg[q].col0 != npad || seg[q].ncol % 32 != 0 || seg[q].k < 1 || seg[q].k > seg[q].ncol ||
@@ -1222,13 +1225,11 @@ cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const Cod
     for (int q = 0; q < nseg; ++q) a.seg[q] = seg[q];
     const long long grid = a.ntiles < sms ? a.ntiles : sms;
     if (nseg == 1) {
-        e = cudaFuncSetAttribute(assign_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+        auto kernel = second.first ? assign_tc_kernel<false, false, true> : assign_tc_kernel<false, false>;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        {
-        const cudaError_t le_ = launch_pdl(assign_tc_kernel<false, false>, dim3((unsigned)grid), dim3(NT), smem, s, tmA, tmBhi, tmBlo, a);
-        if (le_ != cudaSuccess) return le_;
-    }
+        e = launch_pdl(kernel, dim3((unsigned)grid), dim3(NT), smem, s, tmA, tmBhi, tmBlo, a);
+        if (e != cudaSuccess) return e;
     } else {
         e = cudaFuncSetAttribute(assign_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
