@@ -524,7 +524,7 @@ def roofline_score(cfg, kernel_ms, peaks, tcounts=None):
     tbytes = (cfg["H"] + 1) * (cfg["W"] + 1) * k * 2 + V * 4
     hbm = tbytes / (kernel_ms * 1e-3) / 1e9
     out = {"bound": "alu", "achieved": round(ach, 2), "peak": round(peak, 2), "unit": "Tops/s",
-           "frac": round(ach / peak, 4), "traffic": None, "kernel": "score_grid_kernel",
+           "frac": round(ach / peak, 4), "traffic": None, "kernel": "score_grid_tile_kernel",
            "kernel_ms": round(float(kernel_ms), 4),
            "algorithmic_ops_per_window_cluster": round(ops_per, 2),
            "ops_counted": "only the (filter, cluster) pairs with a nonzero template count (the kernel's "
@@ -570,7 +570,7 @@ def run_paper_bank(vq, pipe, cfg, s, dev, reps=5):
     kern = sorted(e[1].elapsed_time(e[2]) for e in ev[1:])[reps // 2]
     return {"bank": "F_{2,3-rect}, S=3 (15 filters, 33 rectangles), equal-weight Gaussian reading",
             "score_call_ms": round(call, 4), "score_kernel_ms": round(kern, 4),
-            "argmax_yx": am.cpu().tolist(), "kernel": "score_wgrid_kernel (weighted 3 x 3 grids, one per sub-scale)"}
+            "argmax_yx": am.cpu().tolist(), "kernel": "score_wgrid_tile_kernel (weighted 3 x 3 grids, one per sub-scale)"}
 
 
 def run_soft(vq, dev, reps=3, B=8):
