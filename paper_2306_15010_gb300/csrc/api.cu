@@ -22,6 +22,12 @@ cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 // ----------------------------------------------------------------------------------
 // Workspace layouts (the same code computes sizes with a null base).
 // ----------------------------------------------------------------------------------
+// Whether an FP8 assignment may take the BF16 second pass.  Below 2^20 feature values its launch and
+// bounds (8 us) cost more than re-scoring, which the chip then does in about one wave: Lloyd steps of a
+// 16 x 19 template, D = 160, take 25 us without it and 33 us with it; from there on re-scoring grows
+// with n D (10 steps, 128 x 128, D = 64: 720 us without it, 428 us with it).
+bool second_pass_pays(long long n, int D) { return n * D >= (1ll << 20); }
+
 AssignWs carve_assign(WsCursor &c, long long n, int D, int k, int prec)
 {
     AssignWs w;
@@ -41,10 +47,9 @@ AssignWs carve_assign(WsCursor &c, long long n, int D, int k, int prec)
     if (prec == VQNNF_PREC_FP8) {
         w.prep.cq8 = c.take<uint8_t>((size_t)k * D);
         w.prep.csc = c.take<float>((size_t)k);
-        if (c.base) {                          // D >= 16: the FP32 copy's storage holds both
-            w.prep.a2 = w.prep.cc;
-            w.prep.v2 = w.prep.cc + k;
-        }
+        const bool second = c.base && second_pass_pays(n, D);
+        w.prep.a2 = second ? w.prep.cc : nullptr;   // D >= 16: the FP32 copy's storage holds both
+        w.prep.v2 = second ? w.prep.cc + k : nullptr;
         w.f8.q = c.take<uint8_t>((size_t)n * D);
         w.f8.rs = c.take<float2>((size_t)n);
     }
@@ -172,11 +177,9 @@ vqnnf_status run_assign(const float *X, long long n, int D, const float *C, int 
     // candidates each; re-scoring streams a centroid per candidate from L2.  Above an eighth of the
     // pixels the BF16 contraction, whose bound leaves 2 %, decides first: it costs one more pass over
     // the features (1024 x 1024, D = 1024, k = 128, 70 % ambiguous: 0.9 ms, re-scoring all of them
-    // 10.6 ms; an eighth of the pixels at 20 candidates re-score in 1.9 ms, at 8 in 0.8 ms).  Where n D
-    // is below 2^21 the launch alone (7 us) costs more than re-scoring, which the chip then does in
-    // about one wave (a 16 x 19 template, D = 160: 25 us per Lloyd step without it, 33 us with it).
+    // 10.6 ms; an eighth of the pixels at 20 candidates re-score in 1.9 ms, at 8 in 0.8 ms).
     SecondPass second = {};
-    if (e == cudaSuccess && prec == VQNNF_PREC_FP8 && n * D >= (1ll << 21)) {
+    if (e == cudaSuccess && prec == VQNNF_PREC_FP8 && w.prep.a2 && second_pass_pays(n, D)) {
         CodebookPrep p = w.prep;
         p.a = w.prep.a2;
         p.v = w.prep.v2;

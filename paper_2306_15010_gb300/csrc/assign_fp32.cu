@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
             v = 2.0 * nc;
             p.csc[j] = csc;
         }
-        if (prec != VQNNF_PREC_FP32) {
+        if (prec == VQNNF_PREC_BF16 || (prec == VQNNF_PREC_FP8 && p.a2)) {
             // Three BF16 products x_hi.hi + x_hi.lo + x_lo.hi.  Tensor-core accumulation
             // order and rounding are not documented: take four times the sequential FP32
             // bound.  The x_lo terms (||x_lo|| <= 2^-8 ||x_hi||) are folded into a_j:

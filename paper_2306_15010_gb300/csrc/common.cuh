@@ -24,7 +24,7 @@ struct CodebookPrep {
     float *b;         // k       bound constant (error of nrm)
     uint8_t *cq8;     // k x D   FP8 e4m3 of (c_j - m) / s_j                 (FP8 path)
     float *csc;       // k       the power-of-two scale s_j                  (FP8 path)
-    float *a2, *v2;   // k       a and v of the BF16 contraction             (FP8 path, second pass)
+    float *a2, *v2;   // k       a and v of the BF16 contraction             (FP8 path; null: no second pass)
 };
 
 // FP8 path: the features quantised per row (x - m = s_x q + residual, s_x a power of two).
