@@ -203,9 +203,6 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
         const double nc = sqrt((c2 + en) * up) * margin;        // ||c*||
         const double ncc = sqrt((double)tot[3] * up) * margin;  // ||fl32(c*)||
         const double nd32 = sqrt((double)tot[4] * up) * margin; // ||c* - fl32(c*)||
-        const double nhi = sqrt((double)tot[5] * up) * margin;
-        const double nlo = sqrt((double)tot[6] * up) * margin;
-        const double nd16 = sqrt((double)tot[7] * up) * margin;
         double a = 0.0, v = 0.0;
         if (prec == VQNNF_PREC_FP32) {
             const double gD = (double)D * u / (1.0 - (double)D * u);
@@ -233,6 +230,9 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
             // order and rounding are not documented: take four times the sequential FP32
             // bound.  The x_lo terms (||x_lo|| <= 2^-8 ||x_hi||) are folded into a_j:
             //   |err| <= X [gacc (|hi| + |lo|) + |d|] + X_lo [gacc |hi| + |lo| + |d|] + ...
+            const double nhi = sqrt((double)tot[5] * up) * margin;
+            const double nlo = sqrt((double)tot[6] * up) * margin;
+            const double nd16 = sqrt((double)tot[7] * up) * margin;
             const double gacc = (double)D * 4.0 * u;
             const double a16 = 2.0 * (gacc * (nhi + nlo) + nd16) + 2.0 * 0.00390625 * (gacc * nhi + nlo + nd16);
             if (prec == VQNNF_PREC_FP8) {
