@@ -111,7 +111,8 @@ enum {
  *   FIT:              H x W = template h x w, D, k, prec
  *   ASSIGN:           H x W pixels, D, k, prec
  *   FILTER_RESPONSES: nothing (returns a small constant)
- *   SCORE:            H x W query, k, th x tw template, F filters
+ *   SCORE:            H x W query, k, th x tw template, F filters; with the same template a
+ *                     smaller H, W or k never needs more
  * Returns 0 for arguments that are out of range. */
 size_t vqnnf_workspace_bytes(int op, int H, int W, int D, int k, int th, int tw, int F,
                              int prec);

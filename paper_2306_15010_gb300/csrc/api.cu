@@ -81,7 +81,7 @@ ScoreWs carve_score(WsCursor &c, int H, int W, int k, int th, int tw)
     const size_t elems = (size_t)(H + 1) * k * sat_pitch(W) + sat_slack_elems(tw);
     w.S = w.u16 ? (void *)c.take<uint16_t>(elems) : (void *)c.take<uint32_t>(elems);
     w.carry = c.take<int>((size_t)H * sat_strips(W) * k);
-    w.bandsum = c.take<int>((size_t)sat_bands(H, W, k) * k * sat_pitch(W));
+    w.bandsum = c.take<int>(sat_bandsum_elems(H, W, k));
     const size_t coarse = (size_t)sat_coarse_rows(H) * sat_coarse_cols(W) * sat_coarse_pitch(k);
     w.coarse = w.u16 ? (void *)c.take<uint16_t>(coarse) : (void *)c.take<uint32_t>(coarse);
     w.aux = c.take<ScoreAux>(1);

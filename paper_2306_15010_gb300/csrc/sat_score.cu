@@ -29,6 +29,7 @@
 // completing on an mbarrier, four buffers in flight); each thread owns four windows and
 // accumulates exact integer L1 distances per filter over all clusters, then combines them
 // in float32 in a fixed filter order.
+#include <algorithm>
 #include <cfloat>
 
 #include "common.cuh"
@@ -645,16 +646,28 @@ int sat_strips(int W) { return (W + 1 + SW - 1) / SW; }
 // Rows of a band: 64, halved (down to 8) while the write pass has fewer than eight warps per SM -- it
 // sweeps a band's rows one after another, and so few warps leave it waiting for memory (256 x 256,
 // k = 16: 20 warps of 64 rows took 62 us, the table 75 us; 25 us in all with bands of 8 rows).
+constexpr int kSatBandWarps = 1216;
 int sat_band_rows(int H, int W, int k)
 {
     int bh = 64;
-    while (bh > 8 && (long long)((H + bh - 1) / bh) * sat_strips(W) * ((k + 31) / 32) < 1216) bh /= 2;
+    while (bh > 8 && (long long)((H + bh - 1) / bh) * sat_strips(W) * ((k + 31) / 32) < kSatBandWarps) bh /= 2;
     return bh;
 }
 int sat_bands(int H, int W, int k)
 {
     const int bh = sat_band_rows(H, W, k);
     return (H + bh - 1) / bh;
+}
+// Room for the band sums of this image and of every smaller one, so that a workspace made for a larger
+// query serves a smaller one whose bands are shorter.  Bands of 64 rows: their number grows with the
+// image.  Shorter ones: at most what bands of 8 rows take, and at most twice the warps of the rule above,
+// less one, of 32 planes x 64 columns each (19.9 MB): twice the height would have had fewer warps than it.
+size_t sat_bandsum_elems(int H, int W, int k)
+{
+    const size_t row = (size_t)k * sat_pitch(W);
+    const size_t tall = (size_t)((H + 63) / 64) * row, low = (size_t)((H + 7) / 8) * row;
+    const size_t most = (size_t)2 * (kSatBandWarps - 1) * 32 * SW;
+    return std::max(tall, std::min(low, most));
 }
 int score_ncol(int tw) { return (TXW + tw + 7) / 8 * 8; }
 size_t sat_slack_elems(int tw) { return (size_t)score_ncol(tw) + 64; }

@@ -78,6 +78,7 @@ int sat_pitch(int W);
 int sat_strips(int W);
 int sat_band_rows(int H, int W, int k);
 int sat_bands(int H, int W, int k);
+size_t sat_bandsum_elems(int H, int W, int k);   // workspace: at least sat_bands * k * sat_pitch, never more for a smaller image
 // Tensor map of the integral image for the write pass: 32 planes x 128 bytes of one row (assign_tc.cu,
 // beside the other maps).
 cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int rows);
