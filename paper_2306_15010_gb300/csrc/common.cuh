@@ -117,6 +117,17 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Lifts the kernel's limit on dynamic shared memory to all that a block can have beside `fixed` bytes of
+// static shared memory.  The limit belongs to the function and not to the launch, so every launch sets the
+// same one: one that set its own size could take the room from another host thread between that thread's
+// setting and its launch.
+constexpr size_t kBlockSmem = 227 * 1024;
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t fixed = 0)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockSmem - fixed));
+}
+
 // Records the caller's profiling event `which` (0 = start, 1 = stop) of operation `op` on s,
 // when vqnnf_set_kernel_events has set one; otherwise does nothing.
 cudaError_t record_kernel_event(int op, int which, cudaStream_t s);

@@ -540,16 +540,14 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
     dim3 grid((WO + TXW - 1) / TXW, HO);
     cudaError_t e;
     if (gs.ncol <= TXW + 128) {
-        e = cudaFuncSetAttribute(score_grid_kernel<T, G, FULL, TXW + 128>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 128>);
         if (e != cudaSuccess) return e;
         {
         const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 128>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
         if (le_ != cudaSuccess) return le_;
     }
     } else {
-        e = cudaFuncSetAttribute(score_grid_kernel<T, G, FULL, TXW + 256>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 256>);
         if (e != cudaSuccess) return e;
         {
         const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 256>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
@@ -567,15 +565,14 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
     const int P = sat_pitch(W);
     const int BH = sat_band_rows(H, W, k), nB = sat_bands(H, W, k);
     const size_t hsmem = sizeof(int) * (size_t)nS * k;
-    cudaError_t e = cudaFuncSetAttribute(row_carry_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsmem);
+    cudaError_t e = allow_smem(row_carry_kernel);
     if (e != cudaSuccess) return e;
     {
         const cudaError_t le_ = launch_pdl(row_carry_kernel, dim3(H), dim3(256), hsmem, s, lab, W, k, nS, carry);
         if (le_ != cudaSuccess) return le_;
     }
     const size_t csmem = sizeof(int) * ((size_t)SW * k + k);
-    e = cudaFuncSetAttribute(band_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem);
+    e = allow_smem(band_sum_kernel);
     if (e != cudaSuccess) return e;
     {
         const cudaError_t le_ = launch_pdl(band_sum_kernel, dim3(dim3(nS, nB)), dim3(256), csmem, s, lab, H, W, k, P, nS, BH, carry, bandsum);
@@ -591,7 +588,7 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
     CUtensorMap map;
     e = make_sat_map(&map, S, sizeof(T) == 2, P, k, H + 1);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(sat_write_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SatTile<T>::smem);
+    e = allow_smem(sat_write_kernel<T>);
     if (e != cudaSuccess) return e;
     e = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * kSatWarps), SatTile<T>::smem, s, map, lab, H, W, k, P, nS, nB,
                    BH, carry, bandsum, coarse);

@@ -671,7 +671,7 @@ cudaError_t launch_wgrid(const Sat<T> &sat, int HO, int WO, const WGridSpec &ws,
     const int nch = WTile<T>::chunks(w);
     const size_t smem = TW * WNST * WTile<T>::stage(nch);
     auto kernel = sep ? score_wgrid_tile_kernel<T, true> : score_wgrid_tile_kernel<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, sizeof(uint16_t) * TW * kMaxWGrids * kMaxK);
     if (e != cudaSuccess) return e;
     return launch_pdl(kernel, dim3((WO + 32 * kWX * TW - 1) / (32 * kWX * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), smem, s, sat,
                       HO, WO, ws, test, nch, tc, heat, amax);
