@@ -128,14 +128,15 @@ __device__ __forceinline__ void warp_argmax(unsigned long long best, unsigned lo
     if ((threadIdx.x & 31) == 0 && best) atomicMax(amax, best);
 }
 
-// Writes this lane's column of the tile; the larger of `best` and its values' keys.
+// Writes this lane's column of the tile, its first `rows` rows; the larger of `best` and its values' keys.
 template <int TY>
 __device__ __forceinline__ unsigned long long put_tile(const float (&hs)[TY], int X, int Y0, int WO,
-                                                       float *__restrict__ heat, unsigned long long best)
+                                                       float *__restrict__ heat, unsigned long long best, int rows = TY)
 {
     if (X < WO) {
 #pragma unroll
         for (int r = 0; r < TY; ++r) {
+            if (r >= rows) break;                            // uniform
             const unsigned idx = (unsigned)((Y0 + r) * WO + X);
             heat[idx] = -hs[r];
             const unsigned long long key = pack_key(-hs[r], idx);
@@ -372,12 +373,13 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
     const int k = sat.k, NG = ws.NG;
     const int X0 = ((int)blockIdx.x * TW + wi) * 32 * NX;
     if (X0 >= WO) return;
-    const int Y0 = min((int)blockIdx.y * TY, HO - TY);
+    const int rows = min(TY, HO);                            // fewer window rows than a tile: the last one repeated
+    const int Y0 = min((int)blockIdx.y * TY, HO - rows);
     const int xe = min(X0 + 32 * NX - 1, WO - 1);
     uint16_t *list = list_s[wi];                             // grid << 8 | cluster, grid by grid
     int n = 0;
     for (int g = 0; g < NG; ++g) {
-        const Region<T> reg(sat, X0 + ws.bx[g][0], Y0 + ws.by[g][0], xe + ws.bx[g][3], Y0 + TY - 1 + ws.by[g][3]);
+        const Region<T> reg(sat, X0 + ws.bx[g][0], Y0 + ws.by[g][0], xe + ws.bx[g][3], Y0 + rows - 1 + ws.by[g][3]);
         for (int j0 = 0; j0 < k; j0 += 128) {
             const int j = j0 + 4 * lane;
             const unsigned h = j >= k ? 0u : (test >> g) & 1 ? reg.holds4(j) : 15u;
@@ -404,7 +406,7 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
                 const int xa = (X0 + ws.bx[g][0]) & ~(E - 1);
                 // chunks up to the last corner column; none starts past the table's row
                 nc = (min(X0 + 32 * NX - 1 + ws.bx[g][3], sat.P - 1) - xa) / E + 1;
-                row = sat.S + (size_t)(Y0 + ws.by[g][lane >> 3] + ((lane >> 1) & 3)) * k * sat.P + xa + (lane & 1) * E;
+                row = sat.S + (size_t)(Y0 + ws.by[g][lane >> 3] + min((lane >> 1) & 3, rows - 1)) * k * sat.P + xa + (lane & 1) * E;
             }
             const uint32_t st = st0 + (uint32_t)ib * stage;
             uint32_t dst = st + (uint32_t)((lane >> 1) * nch + (lane & 1)) * 16;
@@ -532,13 +534,12 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
     }
     unsigned long long best = 0ull;
 #pragma unroll
-    for (int c = 0; c < NX; ++c) best = put_tile<TY>(hs[c], X0 + 32 * c + lane, Y0, WO, heat, best);
+    for (int c = 0; c < NX; ++c) best = put_tile<TY>(hs[c], X0 + 32 * c + lane, Y0, WO, heat, best, rows);
     warp_argmax(best, amax);
 }
 
-// Any bank (weighted half-open rectangles, filter by filter), and the weighted grids of images with
-// fewer than kWY window rows: corners straight from global memory.  Sums in 64 bits: only each
-// filter's counts are known to fit 32.
+// Any bank (weighted half-open rectangles, filter by filter): corners straight from global memory.
+// Sums in 64 bits: only each filter's counts are known to fit 32.
 template <typename T, int TY>
 __global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int HO, int WO, BankSpec bs,
                                                                 const int32_t *__restrict__ tcounts,
@@ -692,11 +693,10 @@ cudaError_t launch_tiles_t(const Sat<T> &sat, int HO, int WO, const BankSpec &bs
     if (gs.G > 0)
         return launch_pdl(score_grid_tile_kernel<T, 2, kGridY>, dim3((WO + 64 * TW - 1) / (64 * TW), (HO + kGridY - 1) / kGridY), dim3(32 * TW),
                           0, s, sat, HO, WO, gs, slot_tests<T>(gs, 64, kGridY), heat, aux, dense_from);
-    if (HO >= kWY) {
-        if (ws.NG > 0) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
+    if (ws.NG > 0) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
+    if (HO >= 4)
         return launch_pdl(score_generic_kernel<T, 4>, dim3((WO + 32 * TW - 1) / (32 * TW), (HO + 3) / 4), dim3(32 * TW), 0, s,
                           sat, HO, WO, bs, tc, heat, amax);
-    }
     return launch_pdl(score_generic_kernel<T, 1>, dim3((WO + 32 * TW - 1) / (32 * TW), HO), dim3(32 * TW), 0, s, sat, HO, WO,
                       bs, tc, heat, amax);
 }
