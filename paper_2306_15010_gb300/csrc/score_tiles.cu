@@ -339,43 +339,56 @@ __global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 14 : 1) score_grid_t
 }
 
 // Weighted-grid bank (WGridSpec): grid by grid, the clusters present in the grid's box add
-// |t - R| - |t| to a filter's sum_j |t_j|, R the filter's integer weighting of the cell counts.
-// Where every filter weights whole columns or whole rows of cells (the Gaussian and Haar filters
-// with equal bin weights: SEP), the three column and three row counts come from the 12 corners on
-// the box's edge; otherwise the nine cell counts from all 16.  A staged (grid, cluster) is the four
-// boundary rows' TY rows, each from the first boundary column on; two lanes copy a row.
-// On a 720 x 1280 query (k = 128, the paper's 15 filters, 97 x 82 template) 0.28 ms, against 2.25 ms
-// for the kernel that visited every cluster and took all nine cells; with three stages 0.33 ms, with
-// tiles of 64 x 4 windows and the grids unrolled 0.67 ms (fewer warps, instruction cache).  It stays
-// the faster one on labels without any coherence (1.44 against 2.26 ms).
-constexpr int kWX = 1, kWY = 4;    // tile: 32 kWX x kWY windows
+// |t - R|, R the filter's integer weighting of the cell counts, to a filter's sum of the other
+// clusters' |t|.  Where every filter weights whole columns or whole rows of cells (the Gaussian and
+// Haar filters with equal bin weights: SEP), the three column and three row counts come from the 12
+// corners on the box's edge; otherwise the nine cell counts from all 16.
+// Bound by the copies: a staged (grid, cluster) is, for each corner, the 32 columns under it of the
+// tile's four rows, consecutive chunks by consecutive lanes, so that an instruction's 512 bytes lie in
+// few lines.  Calls on a 720 x 1280 query with every cluster in every window (k = 128, the paper's 15
+// filters, templates of 110 x 100 to 110 x 250): 1.47 to 1.63 ms at any width; whole rows from the first
+// boundary to the last, two lanes each, 1.71 to 2.84 ms; the kernel that visited every cluster for 512
+// windows 2.41 to 2.49 ms.  Labels in 12-pixel cells with 2 % noise: 1.26 to 1.36 ms.  32-bit table (700 x
+// 250 template, 900 x 800 query, k = 64): 0.37, 0.69 and 0.47 ms.  With exponential bin weights (all 16
+// corners) 1.81 to 2.02, 1.97 to 2.83 and 2.42 to 2.50 ms; 0.40, 0.69 and 0.48 ms.
+constexpr int kWY = 4;             // tile: 32 x kWY windows
 constexpr int WNST = 2;
-template <typename T>
+// A staged pair: the block of kWY rows at each (boundary row a, boundary column q) that is read, every
+// row 32 columns from a 16-byte boundary on; then the pair's template counts.
+template <typename T, bool SEP>
 struct WTile {
-    static constexpr int E = 16 / (int)sizeof(T);
-    // 16-byte chunks of a staged row for a grid `w` columns wide (any alignment), an even number
-    static int chunks(int w) { return ((w + 32 * kWX + E - 1 + E - 1) / E + 1) / 2 * 2; }
-    // shared-memory bytes of one stage: the rows and the template counts
-    static size_t stage(int ch) { return (size_t)16 * 4 * kWY * ch + 32; }
+    static constexpr int E = 16 / (int)sizeof(T);              // elements of a 16-byte chunk
+    static constexpr int CPR = (32 + E - 2) / E + 1;           // chunks per row
+    static constexpr int NB = SEP ? 12 : 16;                   // SEP: no corner inside the box
+    static constexpr int NCH = NB * kWY * CPR;                 // chunks per pair
+    static constexpr int PER = (NCH + 31) / 32;                // per lane
+    static constexpr int STAGE = NCH * 16 + 32;
+    __host__ __device__ static constexpr int block(int a, int q)
+    {
+        return !SEP ? 4 * a + q : a == 0 ? q : a == 3 ? 8 + q : 2 + 2 * a + (q == 3);
+    }
+    // its inverse
+    __device__ static __forceinline__ int row_of(int b) { return !SEP ? b >> 2 : b < 4 ? 0 : b < 8 ? (b - 2) >> 1 : 3; }
+    __device__ static __forceinline__ int col_of(int b) { return !SEP || b < 4 || b >= 8 ? b & 3 : b & 1 ? 3 : 0; }
 };
 
 template <typename T, bool SEP>
 __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, int HO, int WO, WGridSpec ws, unsigned test,
-                                                                   int nch, const int32_t *__restrict__ tcounts,
+                                                                   const int32_t *__restrict__ tcounts,
                                                                    float *__restrict__ heat, unsigned long long *amax)
 {
-    constexpr int E = WTile<T>::E, NX = kWX, TY = kWY;
-    static_assert(TY == 4, "two lanes copy each of the 4 x TY staged rows");
+    using L = WTile<T, SEP>;
+    constexpr int E = L::E, TY = kWY;
     ptx::pdl_enter();
-    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ __align__(16) uint8_t stage_s[TW][WNST][L::STAGE];
     __shared__ uint16_t list_s[TW][kMaxWGrids * kMaxK];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int k = sat.k, NG = ws.NG;
-    const int X0 = ((int)blockIdx.x * TW + wi) * 32 * NX;
+    const int X0 = ((int)blockIdx.x * TW + wi) * 32;
     if (X0 >= WO) return;
     const int rows = min(TY, HO);                            // fewer window rows than a tile: the last one repeated
     const int Y0 = min((int)blockIdx.y * TY, HO - rows);
-    const int xe = min(X0 + 32 * NX - 1, WO - 1);
+    const int xe = min(X0 + 31, WO - 1);
     uint16_t *list = list_s[wi];                             // grid << 8 | cluster, grid by grid
     int n = 0;
     for (int g = 0; g < NG; ++g) {
@@ -393,132 +406,124 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
         }
     }
     __syncwarp();
-    const uint32_t stage = 16 * 4 * TY * nch + 32;
-    uint8_t *mine = smem + (size_t)wi * WNST * stage;
-    const uint32_t st0 = ptx::smem_u32(mine);
-    int ig = -1, nc = 0, ib = 0;                             // grid of the copies, its chunks per row
-    const T *row = nullptr;
+    // the tile's rows start here; offsets from it in 16-byte units stay below 2^32 (checked on the host)
+    const uint4 *S16 = reinterpret_cast<const uint4 *>(sat.S + (size_t)Y0 * k * sat.P);
+    const uint32_t plane16 = (uint32_t)(sat.P / E);
+    uint32_t off[L::PER];                                    // this lane's chunks of a grid
+    const uint32_t st0 = ptx::smem_u32(stage_s[wi][0]) + lane * 16;
+    int ig = -1, ib = 0;                                     // grid of the copies
     auto issue = [&](int p) {
         if (p < n) {
             const int g = list[p] >> 8, j = list[p] & 255;
             if (g != ig) {
                 ig = g;
-                const int xa = (X0 + ws.bx[g][0]) & ~(E - 1);
-                // chunks up to the last corner column; none starts past the table's row
-                nc = (min(X0 + 32 * NX - 1 + ws.bx[g][3], sat.P - 1) - xa) / E + 1;
-                row = sat.S + (size_t)(Y0 + ws.by[g][lane >> 3] + min((lane >> 1) & 3, rows - 1)) * k * sat.P + xa + (lane & 1) * E;
+#pragma unroll
+                for (int i = 0; i < L::PER; ++i) {
+                    const int idx = min(lane + 32 * i, L::NCH - 1), row = idx / L::CPR, ch = idx % L::CPR;
+                    const int blk = row / TY, r = row % TY;
+                    const int x = min(((X0 + ws.bx[g][L::col_of(blk)]) & ~(E - 1)) + ch * E, sat.P - E);
+                    const int y = ws.by[g][L::row_of(blk)] + min(r, rows - 1);
+                    off[i] = (uint32_t)y * (uint32_t)k * plane16 + (uint32_t)(x / E);
+                }
             }
-            const uint32_t st = st0 + (uint32_t)ib * stage;
-            uint32_t dst = st + (uint32_t)((lane >> 1) * nch + (lane & 1)) * 16;
-            const T *src = row + (size_t)j * sat.P;
-            for (int c = lane & 1; c < nc; c += 2, dst += 32, src += 2 * E) cp16(dst, src);
-            if (lane < ws.nf[g]) cp4(st + 16 * 4 * TY * nch + 4 * lane, tcounts + (size_t)ws.filt[g][lane] * k + j);
+            const uint4 *src = S16 + (uint32_t)j * plane16;
+            const uint32_t dst = st0 + (uint32_t)ib * L::STAGE;
+#pragma unroll
+            for (int i = 0; i < L::PER; ++i)
+                if (32 * i + 32 <= L::NCH || lane + 32 * i < L::NCH) cp16(dst + 32 * 16 * i, src + off[i]);
+            if (lane < ws.nf[g]) cp4(dst - lane * 12 + 16 * L::NCH, tcounts + (size_t)ws.filt[g][lane] * k + j);
         }
         cp_commit();
         ib = ib + 1 < WNST ? ib + 1 : 0;
     };
-    float hs[NX][TY];
+    float hs[TY];
 #pragma unroll
-    for (int c = 0; c < NX; ++c)
-#pragma unroll
-        for (int r = 0; r < TY; ++r) hs[c][r] = 0.f;
+    for (int r = 0; r < TY; ++r) hs[r] = 0.f;
 #pragma unroll
     for (int p = 0; p < WNST - 1; ++p) issue(p);
     int p = 0, b = 0;
-    const int rp = nch * E, d = TY * rp;                     // elements to the next staged row, to the next boundary row
 #pragma unroll 1
     for (int g = 0; g < NG; ++g) {
         const int nf = ws.nf[g];
-        int acc[kMaxWFilters][NX][TY];
+        int acc[kMaxWFilters][TY];                           // |t| of the clusters not visited, then |t - R| of the others
 #pragma unroll
         for (int f = 0; f < kMaxWFilters; ++f) {
             int ts = 0;
             if (f < nf) {
                 const int32_t *tc = tcounts + (size_t)ws.filt[g][f] * k;
                 for (int j = lane; j < k; j += 32) ts += abs(tc[j]);
+                for (int q = p + lane; q < n && (list[q] >> 8) == g; q += 32) ts -= abs(tc[list[q] & 255]);
                 ts = __reduce_add_sync(0xffffffffu, ts);
             }
 #pragma unroll
-            for (int c = 0; c < NX; ++c)
-#pragma unroll
-                for (int r = 0; r < TY; ++r) acc[f][c][r] = ts;
+            for (int r = 0; r < TY; ++r) acc[f][r] = ts;
         }
         int col[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) col[c] = lane + ws.bx[g][c] - ws.bx[g][0] + ((X0 + ws.bx[g][0]) & (E - 1));
+        for (int q = 0; q < 4; ++q) col[q] = lane + ((X0 + ws.bx[g][q]) & (E - 1));
 #pragma unroll 1
         for (; p < n && (list[p] >> 8) == g; ++p) {
             cp_wait<WNST - 2>();
             __syncwarp();
             issue(p + WNST - 1);
-            const T *v = reinterpret_cast<const T *>(mine + (size_t)b * stage);
-            const int *ts = reinterpret_cast<const int *>(mine + (size_t)b * stage + 16 * 4 * TY * nch);
+            const T *v = reinterpret_cast<const T *>(stage_s[wi][b]);
+            const int *ts = reinterpret_cast<const int *>(stage_s[wi][b] + 16 * L::NCH);
             constexpr int NN = SEP ? 6 : 9;
-            int m[NX][TY][NN];                               // column and row counts, or cell counts
+            int m[TY][NN];                                   // column and row counts, or cell counts
+            auto at = [&](int a, int q, int r) { return (int)v[(L::block(a, q) * TY + r) * L::CPR * E + col[q]]; };
 #pragma unroll
-            for (int r = 0; r < TY; ++r)
+            for (int r = 0; r < TY; ++r) {
+                if (SEP) {
+                    int top[4], bot[4], lft[4], rgt[4];
 #pragma unroll
-                for (int c = 0; c < NX; ++c) {
-                    const T *e = v + r * rp + 32 * c;
-                    if (SEP) {
-                        int top[4], bot[4], lft[4], rgt[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            top[i] = (int)e[col[i]];
-                            bot[i] = (int)e[3 * d + col[i]];
-                        }
-                        lft[0] = top[0], rgt[0] = top[3], lft[3] = bot[0], rgt[3] = bot[3];
-#pragma unroll
-                        for (int i = 1; i < 3; ++i) {
-                            lft[i] = (int)e[i * d + col[0]];
-                            rgt[i] = (int)e[i * d + col[3]];
-                        }
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) {
-                            m[c][r][i] = box<T>(bot[i + 1], bot[i], top[i + 1], top[i]);
-                            m[c][r][3 + i] = box<T>(rgt[i + 1], lft[i + 1], rgt[i], lft[i]);
-                        }
-                    } else {
-                        int cr[4][4];
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) cr[a][i] = (int)e[a * d + col[i]];
-#pragma unroll
-                        for (int a = 0; a < 3; ++a)
-#pragma unroll
-                            for (int i = 0; i < 3; ++i)
-                                m[c][r][(a * 3 + i) % NN] = box<T>(cr[a + 1][i + 1], cr[a + 1][i], cr[a][i + 1], cr[a][i]);
+                    for (int i = 0; i < 4; ++i) {
+                        top[i] = at(0, i, r);
+                        bot[i] = at(3, i, r);
+                        lft[i] = at(i, 0, r);
+                        rgt[i] = at(i, 3, r);
                     }
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        m[r][i] = box<T>(bot[i + 1], bot[i], top[i + 1], top[i]);
+                        m[r][3 + i] = box<T>(rgt[i + 1], lft[i + 1], rgt[i], lft[i]);
+                    }
+                } else {
+                    int cr[4][4];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) cr[a][i] = at(a, i, r);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int i = 0; i < 3; ++i)
+                            m[r][(a * 3 + i) % NN] = box<T>(cr[a + 1][i + 1], cr[a + 1][i], cr[a][i + 1], cr[a][i]);
                 }
+            }
 #pragma unroll
             for (int f = 0; f < kMaxWFilters; ++f) {
                 if (f >= nf) break;
-                const int t = ts[f], at = abs(t);
-                if (SEP && ws.rowwise[g][f]) {
-                    const int w0 = ws.w[g][f][0], w1 = ws.w[g][f][3], w2 = ws.w[g][f][6];
-#pragma unroll
-                    for (int c = 0; c < NX; ++c)
-#pragma unroll
-                        for (int r = 0; r < TY; ++r)
-                            acc[f][c][r] += abs(t - (w0 * m[c][r][3] + w1 * m[c][r][4] + w2 * m[c][r][5])) - at;
-                } else if (SEP) {
-                    const int w0 = ws.w[g][f][0], w1 = ws.w[g][f][1], w2 = ws.w[g][f][2];
-#pragma unroll
-                    for (int c = 0; c < NX; ++c)
+                const int t = ts[f];
+                if (SEP) {
+                    const bool rowwise = ws.rowwise[g][f];
+                    const int w0 = ws.w[g][f][0], w1 = ws.w[g][f][rowwise ? 3 : 1], w2 = ws.w[g][f][rowwise ? 6 : 2];
+                    if (rowwise) {
 #pragma unroll
                         for (int r = 0; r < TY; ++r)
-                            acc[f][c][r] += abs(t - (w0 * m[c][r][0] + w1 * m[c][r][1] + w2 * m[c][r][2])) - at;
+                            acc[f][r] = (int)__sad(t, w0 * m[r][3] + w1 * m[r][4] + w2 * m[r][5], (unsigned)acc[f][r]);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < TY; ++r)
+                            acc[f][r] = (int)__sad(t, w0 * m[r][0] + w1 * m[r][1] + w2 * m[r][2], (unsigned)acc[f][r]);
+                    }
                 } else {
 #pragma unroll
-                    for (int c = 0; c < NX; ++c)
+                    for (int r = 0; r < TY; ++r) {
+                        int R = 0;
 #pragma unroll
-                        for (int r = 0; r < TY; ++r) {
-                            int R = 0;
-#pragma unroll
-                            for (int i = 0; i < 9; ++i) R += ws.w[g][f][i] * m[c][r][i % NN];
-                            acc[f][c][r] += abs(t - R) - at;
-                        }
+                        for (int i = 0; i < 9; ++i) R += ws.w[g][f][i] * m[r][i % NN];
+                        acc[f][r] = (int)__sad(t, R, (unsigned)acc[f][r]);
+                    }
                 }
             }
             b = b + 1 < WNST ? b + 1 : 0;
@@ -527,15 +532,10 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
         for (int f = 0; f < kMaxWFilters; ++f) {
             if (f >= nf) break;
 #pragma unroll
-            for (int c = 0; c < NX; ++c)
-#pragma unroll
-                for (int r = 0; r < TY; ++r) hs[c][r] = fmaf(ws.coef[g][f], (float)acc[f][c][r], hs[c][r]);
+            for (int r = 0; r < TY; ++r) hs[r] = fmaf(ws.coef[g][f], (float)acc[f][r], hs[r]);
         }
     }
-    unsigned long long best = 0ull;
-#pragma unroll
-    for (int c = 0; c < NX; ++c) best = put_tile<TY>(hs[c], X0 + 32 * c + lane, Y0, WO, heat, best, rows);
-    warp_argmax(best, amax);
+    warp_argmax(put_tile<TY>(hs, X0 + lane, Y0, WO, heat, 0ull, rows), amax);
 }
 
 // Any bank (weighted half-open rectangles, filter by filter): corners straight from global memory.
@@ -656,26 +656,28 @@ unsigned slot_tests(const GridSpec &gs, int w, int h)
     return test;
 }
 
+// A weighted-grid bank whose tiles' rows are within 32-bit offsets in 16-byte units (a table of 64 GiB or
+// more under the template's rows is not; such a bank goes filter by filter).
+bool wgrid_fits(const WGridSpec &ws, int k, int plane16)
+{
+    int h = 0;
+    for (int g = 0; g < ws.NG; ++g) h = ws.by[g][3] > h ? ws.by[g][3] : h;
+    return ws.NG > 0 && (long long)(h + kWY) * k * plane16 < (1ll << 32);
+}
+
 template <typename T>
 cudaError_t launch_wgrid(const Sat<T> &sat, int HO, int WO, const WGridSpec &ws, const int32_t *tc, float *heat,
                          unsigned long long *amax, cudaStream_t s)
 {
     unsigned test = 0;
-    int w = 0;
     bool sep = true;
     for (int g = 0; g < ws.NG; ++g) {
-        const int gw = ws.bx[g][3] - ws.bx[g][0];
-        w = gw > w ? gw : w;
         sep = sep && ws.sep[g];
-        test |= (unsigned)testable<T>(gw + 32 * kWX - 1, ws.by[g][3] - ws.by[g][0] + kWY - 1) << g;
+        test |= (unsigned)testable<T>(ws.bx[g][3] - ws.bx[g][0] + 31, ws.by[g][3] - ws.by[g][0] + kWY - 1) << g;
     }
-    const int nch = WTile<T>::chunks(w);
-    const size_t smem = TW * WNST * WTile<T>::stage(nch);
-    auto kernel = sep ? score_wgrid_tile_kernel<T, true> : score_wgrid_tile_kernel<T, false>;
-    cudaError_t e = allow_smem(kernel, sizeof(uint16_t) * TW * kMaxWGrids * kMaxK);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(kernel, dim3((WO + 32 * kWX * TW - 1) / (32 * kWX * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), smem, s, sat,
-                      HO, WO, ws, test, nch, tc, heat, amax);
+    return launch_pdl(sep ? score_wgrid_tile_kernel<T, true> : score_wgrid_tile_kernel<T, false>,
+                      dim3((WO + 32 * TW - 1) / (32 * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), 0, s, sat, HO, WO, ws, test, tc,
+                      heat, amax);
 }
 
 template <typename T>
@@ -693,7 +695,7 @@ cudaError_t launch_tiles_t(const Sat<T> &sat, int HO, int WO, const BankSpec &bs
     if (gs.G > 0)
         return launch_pdl(score_grid_tile_kernel<T, 2, kGridY>, dim3((WO + 64 * TW - 1) / (64 * TW), (HO + kGridY - 1) / kGridY), dim3(32 * TW),
                           0, s, sat, HO, WO, gs, slot_tests<T>(gs, 64, kGridY), heat, aux, dense_from);
-    if (ws.NG > 0) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
+    if (wgrid_fits(ws, sat.k, sat.P / WTile<T, true>::E)) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
     if (HO >= 4)
         return launch_pdl(score_generic_kernel<T, 4>, dim3((WO + 32 * TW - 1) / (32 * TW), (HO + 3) / 4), dim3(32 * TW), 0, s,
                           sat, HO, WO, bs, tc, heat, amax);
