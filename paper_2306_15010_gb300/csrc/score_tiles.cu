@@ -343,33 +343,34 @@ __global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 14 : 1) score_grid_t
 // clusters' |t|.  Where every filter weights whole columns or whole rows of cells (the Gaussian and
 // Haar filters with equal bin weights: SEP), the three column and three row counts come from the 12
 // corners on the box's edge; otherwise the nine cell counts from all 16.
-// Bound by the copies: a staged (grid, cluster) is, for each corner, the 32 columns under it of the
-// tile's four rows, consecutive chunks by consecutive lanes, so that an instruction's 512 bytes lie in
-// few lines.  Calls on a 720 x 1280 query with every cluster in every window (k = 128, the paper's 15
-// filters, templates of 110 x 100 to 110 x 250): 1.47 to 1.63 ms at any width; whole rows from the first
-// boundary to the last, two lanes each, 1.71 to 2.84 ms; the kernel that visited every cluster for 512
-// windows 2.41 to 2.49 ms.  Labels in 12-pixel cells with 2 % noise: 1.26 to 1.36 ms.  32-bit table (700 x
-// 250 template, 900 x 800 query, k = 64): 0.37, 0.69 and 0.47 ms.  With exponential bin weights (all 16
-// corners) 1.81 to 2.02, 1.97 to 2.83 and 2.42 to 2.50 ms; 0.40, 0.69 and 0.48 ms.
+// Bound by the copies: a staged (grid, cluster) is 16 rows, each the 32 columns at every boundary or all
+// columns between, eight lanes to a row, so that an instruction's copies lie in few lines.  Calls on a
+// 720 x 1280 query with every cluster in every window (k = 128, the paper's 15 filters, templates of
+// 110 x 100 to 110 x 250): 1.45 to 1.63 ms at any width; whole rows alone, two lanes each, 1.68 to 2.84 ms;
+// the kernel that visited every cluster for 512 windows 2.41 to 2.49 ms.  Labels in 12-pixel cells with
+// 2 % noise 1.19 to 1.45, 1.37 to 2.51 ms.  32-bit table (700 x 100 to 700 x 250 template, 900 x 800 query,
+// k = 64) 0.33 to 0.39, 0.41 to 0.69 and 0.47 ms.  With exponential bin weights (all 16 corners) 1.72 to
+// 1.88, 2.03 to 2.70 and 2.42 to 2.50 ms; 0.33 to 0.40, 0.40 to 0.70 and 0.48 ms.
 constexpr int kWY = 4;             // tile: 32 x kWY windows
 constexpr int WNST = 2;
-// A staged pair: the block of kWY rows at each (boundary row a, boundary column q) that is read, every
-// row 32 columns from a 16-byte boundary on; then the pair's template counts.
+// A staged pair: kWY rows for each boundary row a, then the pair's template counts.  A row has room for
+// the 32 columns at each boundary column that is read (SEP: the outer two alone in the box's inner rows),
+// each from a 16-byte boundary on; or it holds all columns from the first boundary's to the last's,
+// where these are fewer.
 template <typename T, bool SEP>
 struct WTile {
     static constexpr int E = 16 / (int)sizeof(T);              // elements of a 16-byte chunk
     static constexpr int CPR = (32 + E - 2) / E + 1;           // chunks per row
-    static constexpr int NB = SEP ? 12 : 16;                   // SEP: no corner inside the box
-    static constexpr int NCH = NB * kWY * CPR;                 // chunks per pair
-    static constexpr int PER = (NCH + 31) / 32;                // per lane
+    static constexpr int R0 = 4 * CPR, R1 = SEP ? 2 * CPR : R0;   // chunks of an outer and of an inner row
+    static constexpr int NCH = 2 * kWY * (R0 + R1);            // chunks per pair
     static constexpr int STAGE = NCH * 16 + 32;
-    __host__ __device__ static constexpr int block(int a, int q)
+    // first chunk of boundary row a, tile row r
+    __host__ __device__ static constexpr int row(int a, int r)
     {
-        return !SEP ? 4 * a + q : a == 0 ? q : a == 3 ? 8 + q : 2 + 2 * a + (q == 3);
+        return a == 0 ? r * R0 : a == 3 ? kWY * (R0 + 2 * R1) + r * R0 : kWY * (R0 + (a - 1) * R1) + r * R1;
     }
-    // its inverse
-    __device__ static __forceinline__ int row_of(int b) { return !SEP ? b >> 2 : b < 4 ? 0 : b < 8 ? (b - 2) >> 1 : 3; }
-    __device__ static __forceinline__ int col_of(int b) { return !SEP || b < 4 || b >= 8 ? b & 3 : b & 1 ? 3 : 0; }
+    // chunks of all columns of a grid `w` columns wide
+    __device__ static __forceinline__ int whole(int w) { return (w + 30 + E) / E + 1; }
 };
 
 template <typename T, bool SEP>
@@ -409,29 +410,54 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
     // the tile's rows start here; offsets from it in 16-byte units stay below 2^32 (checked on the host)
     const uint4 *S16 = reinterpret_cast<const uint4 *>(sat.S + (size_t)Y0 * k * sat.P);
     const uint32_t plane16 = (uint32_t)(sat.P / E);
-    uint32_t off[L::PER];                                    // this lane's chunks of a grid
-    const uint32_t st0 = ptx::smem_u32(stage_s[wi][0]) + lane * 16;
-    int ig = -1, ib = 0;                                     // grid of the copies
+    // Eight lanes copy a row (of one a), chunk c, c + 8, ..: an instruction's four rows lie in few lines.
+    // The last chunks may end past the table's row, and past the table by less than its slack.
+    const int c = lane & 7, r0 = lane >> 3;
+    S16 += X0 / E + (uint32_t)min(r0, rows - 1) * (uint32_t)k * plane16 + c;
+    const uint32_t st0 = ptx::smem_u32(stage_s[wi][0]) + 16 * c;
+    int ig = -1, ib = 0, cw = 0;                             // grid of the copies, the chunks of its whole rows
+    int nfg = 0;                                             // its filters, and this lane's filter's counts
+    const int32_t *tcf = tcounts;
+    uint32_t ya[4], xq[4];                                   // its boundary rows and columns, in chunks
     auto issue = [&](int p) {
         if (p < n) {
             const int g = list[p] >> 8, j = list[p] & 255;
             if (g != ig) {
                 ig = g;
+                cw = L::whole(ws.bx[g][3] - ws.bx[g][0]);
+                nfg = ws.nf[g];
+                tcf = tcounts + (size_t)ws.filt[g][min(lane, kMaxWFilters - 1)] * k;
 #pragma unroll
-                for (int i = 0; i < L::PER; ++i) {
-                    const int idx = min(lane + 32 * i, L::NCH - 1), row = idx / L::CPR, ch = idx % L::CPR;
-                    const int blk = row / TY, r = row % TY;
-                    const int x = min(((X0 + ws.bx[g][L::col_of(blk)]) & ~(E - 1)) + ch * E, sat.P - E);
-                    const int y = ws.by[g][L::row_of(blk)] + min(r, rows - 1);
-                    off[i] = (uint32_t)y * (uint32_t)k * plane16 + (uint32_t)(x / E);
+                for (int a = 0; a < 4; ++a) {
+                    ya[a] = (uint32_t)ws.by[g][a] * (uint32_t)k * plane16;
+                    xq[a] = (uint32_t)(ws.bx[g][a] / E);
                 }
             }
             const uint4 *src = S16 + (uint32_t)j * plane16;
             const uint32_t dst = st0 + (uint32_t)ib * L::STAGE;
 #pragma unroll
-            for (int i = 0; i < L::PER; ++i)
-                if (32 * i + 32 <= L::NCH || lane + 32 * i < L::NCH) cp16(dst + 32 * 16 * i, src + off[i]);
-            if (lane < ws.nf[g]) cp4(dst - lane * 12 + 16 * L::NCH, tcounts + (size_t)ws.filt[g][lane] * k + j);
+            for (int a = 0; a < 4; ++a) {
+                const bool outer = a == 0 || a == 3;
+                const int R = outer ? L::R0 : L::R1;
+                const uint4 *from = src + ya[a];
+                const uint32_t to = dst + 16 * (L::row(a, 0) + r0 * R);
+                if (cw <= R) {
+                    from += xq[0];
+#pragma unroll
+                    for (int h = 0; h < R; h += 8)
+                        if (c + h < cw) cp16(to + 16 * h, from + h);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (SEP && !outer && (q == 1 || q == 2)) continue;
+                        const int sg = SEP && !outer ? q / 3 : q;
+#pragma unroll
+                        for (int h = 0; h < L::CPR; h += 8)
+                            if (c + h < L::CPR) cp16(to + 16 * (sg * L::CPR + h), from + (xq[q] + h));
+                    }
+                }
+            }
+            if (lane < nfg) cp4(dst - 16 * c + lane * 4 + 16 * L::NCH, tcf + j);
         }
         cp_commit();
         ib = ib + 1 < WNST ? ib + 1 : 0;
@@ -458,9 +484,16 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
 #pragma unroll
             for (int r = 0; r < TY; ++r) acc[f][r] = ts;
         }
-        int col[4];
+        const int cw = L::whole(ws.bx[g][3] - ws.bx[g][0]);
+        int col[4], last;                                    // places in an outer row, and of the last column in an inner row
+        {
+            const int x0 = X0 + ws.bx[g][0], s0 = x0 & (E - 1), s3 = (X0 + ws.bx[g][3]) & (E - 1);
+            const int end = lane + ws.bx[g][3] - ws.bx[g][0] + s0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) col[q] = lane + ((X0 + ws.bx[g][q]) & (E - 1));
+            for (int q = 0; q < 4; ++q)
+                col[q] = lane + (cw <= L::R0 ? ws.bx[g][q] - ws.bx[g][0] + s0 : q * L::CPR * E + ((X0 + ws.bx[g][q]) & (E - 1)));
+            last = !SEP ? col[3] : cw <= L::R1 ? end : lane + L::CPR * E + s3;
+        }
 #pragma unroll 1
         for (; p < n && (list[p] >> 8) == g; ++p) {
             cp_wait<WNST - 2>();
@@ -470,7 +503,7 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
             const int *ts = reinterpret_cast<const int *>(stage_s[wi][b] + 16 * L::NCH);
             constexpr int NN = SEP ? 6 : 9;
             int m[TY][NN];                                   // column and row counts, or cell counts
-            auto at = [&](int a, int q, int r) { return (int)v[(L::block(a, q) * TY + r) * L::CPR * E + col[q]]; };
+            auto at = [&](int a, int q, int r) { return (int)v[L::row(a, r) * E + (q == 3 && (a == 1 || a == 2) ? last : col[q])]; };
 #pragma unroll
             for (int r = 0; r < TY; ++r) {
                 if (SEP) {
