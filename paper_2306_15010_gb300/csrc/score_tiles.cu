@@ -573,6 +573,15 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
 
 // Any bank (weighted half-open rectangles, filter by filter): corners straight from global memory.
 // Sums in 64 bits: only each filter's counts are known to fit 32.
+// Bound by the corners' loads; a filter's template counts wait in shared memory, since between them the
+// corners leave L1 no room (32-bit table, 1024 x 1024, k = 128, ten filters over a 200 x 400 template:
+// 1.83 ms, read where they are used and their |t| added up by every lane 3.46; the kernel that staged every
+// cluster for 512 windows 3.30).  Tiles of four rows share loads of neighbouring rows' lines, but
+// below 13 of their warps per SM too few are in flight, and one row a warp is faster: 700 x 700, k =
+// 128, 300 x 300 template (1,313 warps) 1.11 against 1.63 ms, 200 x 200, k = 32, ten filters of six
+// rectangles (258) 0.40 against 0.75; 720 x 1280, k = 128, 240 x 250 template (3,993), two filters, 1.20
+// against 0.79.
+constexpr int kGenericWarps = 1976;   // 13 per SM
 template <typename T, int TY>
 __global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int HO, int WO, BankSpec bs,
                                                                 const int32_t *__restrict__ tcounts,
@@ -580,6 +589,7 @@ __global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int 
 {
     ptx::pdl_enter();
     __shared__ unsigned act_s[TW][kMaskWords];
+    __shared__ int tc_s[TW][kMaxK];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int k = sat.k, nw = words_of(k);
     const int X0 = ((int)blockIdx.x * TW + wi) * 32;
@@ -603,7 +613,14 @@ __global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int 
                        Region<T>(sat, X0 + bx0, Y0 + by0, xe + bx1, Y0 + TY - 1 + by1));
         __syncwarp();
         long long ts = 0, acc[TY];
-        for (int j = 0; j < k; ++j) ts += abs(tc[j]);
+        for (int j = lane; j < k; j += 32) {
+            const int t = tc[j];
+            tc_s[wi][j] = t;
+            ts += abs(t);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, o);
 #pragma unroll
         for (int r = 0; r < TY; ++r) acc[r] = ts;
         int w = 0;
@@ -611,7 +628,7 @@ __global__ void __launch_bounds__(32 * TW) score_generic_kernel(Sat<T> sat, int 
         while (true) {
             while (m == 0 && ++w < nw) m = act[w];
             if (m == 0) break;
-            const int j = word_cluster(w, m), t = tc[j];
+            const int j = word_cluster(w, m), t = tc_s[wi][j];
             m &= m - 1;
             const T *base = sat.S + ((size_t)Y0 * k + j) * sat.P + xl;
             int v[TY];
@@ -729,7 +746,7 @@ cudaError_t launch_tiles_t(const Sat<T> &sat, int HO, int WO, const BankSpec &bs
         return launch_pdl(score_grid_tile_kernel<T, 2, kGridY>, dim3((WO + 64 * TW - 1) / (64 * TW), (HO + kGridY - 1) / kGridY), dim3(32 * TW),
                           0, s, sat, HO, WO, gs, slot_tests<T>(gs, 64, kGridY), heat, aux, dense_from);
     if (wgrid_fits(ws, sat.k, sat.P / WTile<T, true>::E)) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
-    if (HO >= 4)
+    if (HO >= 4 && (long long)((WO + 31) / 32) * ((HO + 3) / 4) >= kGenericWarps)
         return launch_pdl(score_generic_kernel<T, 4>, dim3((WO + 32 * TW - 1) / (32 * TW), (HO + 3) / 4), dim3(32 * TW), 0, s,
                           sat, HO, WO, bs, tc, heat, amax);
     return launch_pdl(score_generic_kernel<T, 1>, dim3((WO + 32 * TW - 1) / (32 * TW), HO), dim3(32 * TW), 0, s, sat, HO, WO,
