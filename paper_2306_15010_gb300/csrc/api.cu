@@ -264,7 +264,7 @@ vqnnf_status run_fit(const float *T, long long l, int D, int k, int iters, uint6
 // the box into a 3 x 3 grid (repeated last boundaries give empty cells), every rectangle is a
 // union of whole cells, and each filter becomes its cell weights.  Counts and per-window L1
 // sums must stay inside int32.
-void detect_wgrid(const vqnnf_filter *bank, int F, const BankSpec &bs, WGridSpec &ws)
+void detect_wgrid(const vqnnf_filter *bank, int F, int tw, const BankSpec &bs, WGridSpec &ws)
 {
     memset(&ws, 0, sizeof(ws));
     int gbox[kMaxWGrids][4];
@@ -337,8 +337,7 @@ void detect_wgrid(const vqnnf_filter *bank, int F, const BankSpec &bs, WGridSpec
         }
     }
     ws.NG = ng;
-    ws.ncol = bs.ncol;
-    if (!score_grid_fits(bs.ncol)) ws.NG = 0;
+    if (!score_grid_fits(score_ncol(tw))) ws.NG = 0;
 }
 
 vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankSpec &bs,
@@ -348,8 +347,6 @@ vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankS
     if (F > kMaxFilters) return VQNNF_EUNSUPPORTED;
     memset(&bs, 0, sizeof(bs));
     memset(&gs, 0, sizeof(gs));
-    int nr = 0;
-    int rows[kMaxRows];
     int nrect = 0;
     for (int f = 0; f < F; ++f) {
         const vqnnf_filter &fl = bank[f];
@@ -365,25 +362,12 @@ vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankS
                 return VQNNF_EINVAL;
             RectSpec &o = bs.rect[nrect++];
             o.x0 = rc.x0; o.y0 = rc.y0; o.x1 = rc.x1; o.y1 = rc.y1; o.weight = rc.weight;
-            for (int yy : {rc.y0, rc.y1}) {
-                bool seen = false;
-                for (int q = 0; q < nr; ++q) seen |= rows[q] == yy;
-                if (!seen) rows[nr++] = yy;
-            }
         }
         bs.coef[f] = (float)((double)fl.w_f / (double)fl.area);
     }
     bs.rect_begin[F] = nrect;
     bs.F = F;
-    std::sort(rows, rows + nr);
-    bs.nrow = nr;
-    for (int q = 0; q < nr; ++q) bs.roff[q] = rows[q];
-    for (int r = 0; r < nrect; ++r) {
-        RectSpec &o = bs.rect[r];
-        o.ry0 = int(std::lower_bound(rows, rows + nr, o.y0) - rows);
-        o.ry1 = int(std::lower_bound(rows, rows + nr, o.y1) - rows);
-    }
-    bs.ncol = score_ncol(tw);
+    const int ncol = score_ncol(tw);
 
     // grid detection: single unit-weight rectangles forming a G x G cell grid (+ full)
     bool single = true;
@@ -410,7 +394,7 @@ vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankS
         return VQNNF_OK;
     const int ncell = F - (full_f >= 0 ? 1 : 0);
     if (ncell != G * G) return VQNNF_OK;
-    if (!score_grid_fits(bs.ncol)) return VQNNF_OK;       // template wider than the grid kernel stages
+    if (!score_grid_fits(ncol)) return VQNNF_OK;          // template wider than the grid kernel stages
     int seen[16] = {0};
     GridSpec g;
     memset(&g, 0, sizeof(g));
@@ -431,7 +415,7 @@ vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankS
     g.G = G;
     g.full = full_f >= 0;
     g.F = F;
-    g.ncol = bs.ncol;
+    g.ncol = ncol;
     for (int q = 0; q <= G; ++q) {
         g.bx[q] = xs[q];
         g.by[q] = ys[q];
@@ -445,15 +429,6 @@ vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankS
     }
     gs = g;
     return VQNNF_OK;
-}
-
-int device_smem_optin()
-{
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-        return 0;
-    return v;
 }
 
 }  // namespace vqnnf
@@ -569,10 +544,7 @@ vqnnf_status vqnnf_score(const uint8_t *q_labels, int H, int W, int k, int th, i
     vqnnf_status st = compile_bank(bank, F, th, tw, bs, gs);
     if (st != VQNNF_OK) return st;
     memset(&wg, 0, sizeof(wg));
-    if (gs.G == 0) detect_wgrid(bank, F, bs, wg);
-    const bool u16 = sat_is_u16(th, tw);
-    if (wg.NG == 0 && score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k) > (size_t)device_smem_optin())
-        return VQNNF_EUNSUPPORTED;
+    if (gs.G == 0) detect_wgrid(bank, F, tw, bs, wg);
     cudaStream_t s = as_stream(stream);
     WsCursor c{static_cast<char *>(ws), 0};
     ScoreWs sw = carve_score(c, H, W, k, th, tw);
@@ -619,10 +591,7 @@ vqnnf_status vqnnf_match_host(const float *X_host, int H, int W, int D, const fl
     WGridSpec wg;
     if ((st = compile_bank(bank, F, th, tw, bs, gs)) != VQNNF_OK) return st;
     memset(&wg, 0, sizeof(wg));
-    if (gs.G == 0) detect_wgrid(bank, F, bs, wg);
-    const bool u16 = sat_is_u16(th, tw);
-    if (wg.NG == 0 && score_smem_bytes_for(u16 ? 2 : 4, bs, gs, k) > (size_t)device_smem_optin())
-        return VQNNF_EUNSUPPORTED;
+    if (gs.G == 0) detect_wgrid(bank, F, tw, bs, wg);
     WsCursor cur{static_cast<char *>(ws), 0};
     HostWs w = carve_host(cur, H, W, D, k, th, tw, F, prec);
     const cudaStream_t s = as_stream(stream), cs = stream2 ? as_stream(stream2) : s;

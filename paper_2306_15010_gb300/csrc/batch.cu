@@ -397,13 +397,10 @@ vqnnf_status compile_banks(const vqnnf_batch_template *t, int nt, int G, Banks &
     b.gs.resize(nt);
     std::vector<vqnnf_rect> rects;
     std::vector<vqnnf_filter> bank;
-    const int optin = device_smem_optin();
     for (int j = 0; j < nt; ++j) {
         grid_bank(t[j].h, t[j].w, G, rects, bank);
         vqnnf_status st = compile_bank(bank.data(), (int)bank.size(), t[j].h, t[j].w, b.bs[j], b.gs[j]);
         if (st != VQNNF_OK) return st;
-        const bool u16 = sat_is_u16(t[j].h, t[j].w);
-        if (score_smem_bytes_for(u16 ? 2 : 4, b.bs[j], b.gs[j], t[j].k) > (size_t)optin) return VQNNF_EUNSUPPORTED;
     }
     return VQNNF_OK;
 }

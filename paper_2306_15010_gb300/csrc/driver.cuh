@@ -33,7 +33,6 @@ cudaStream_t as_stream(void *s);
 bool aligned(const void *p, size_t a);
 vqnnf_status from_cuda(cudaError_t e);
 bool check_prec(int prec, int D);
-int device_smem_optin();
 
 AssignWs carve_assign(WsCursor &c, long long n, int D, int k, int prec = VQNNF_PREC_FP32);
 FitWs carve_fit(WsCursor &c, long long l, int D, int k, int prec = VQNNF_PREC_FP32);
@@ -49,6 +48,6 @@ vqnnf_status run_fit(const float *T, long long l, int D, int k, int iters, uint6
                      float *C, FitWs &fw, cudaStream_t s);
 // Host-side description of a filter bank for the score kernels (grid bank detected).
 vqnnf_status compile_bank(const vqnnf_filter *bank, int F, int th, int tw, BankSpec &bs, GridSpec &gs);
-void detect_wgrid(const vqnnf_filter *bank, int F, const BankSpec &bs, WGridSpec &ws);
+void detect_wgrid(const vqnnf_filter *bank, int F, int tw, const BankSpec &bs, WGridSpec &ws);
 
 }  // namespace vqnnf

@@ -529,14 +529,20 @@ __global__ void argmax_finish_kernel(const unsigned long long *amax, int WO, int
     out[1] = (int32_t)(idx % (unsigned)WO);
 }
 
+size_t score_grid_smem(size_t elem, const GridSpec &gs, int k)   // 79 KB at most
+{
+    const int NR = gs.G + 1;
+    const int NSLOT = gs.G * gs.G + (gs.full ? 1 : 0);
+    const int pitch = gs.ncol <= TXW + 128 ? TXW + 128 : TXW + 256;
+    return elem * (size_t)NBUF * CH * NR * pitch + sizeof(int) * ((size_t)NSLOT * k + k + 1) + sizeof(uint64_t) * 2 * NBUF + 16 + 16;
+}
+
 template <typename T, int G, bool FULL>
 cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec &gs, const int32_t *tc,
                         float *heat, unsigned long long *amax, const long long *probe, long long dense_from,
                         cudaStream_t s)
 {
-    BankSpec none;
-    none.F = 0;
-    const size_t smem = score_smem_bytes_for(sizeof(T), none, gs, k);
+    const size_t smem = score_grid_smem(sizeof(T), gs, k);
     dim3 grid((WO + TXW - 1) / TXW, HO);
     cudaError_t e;
     if (gs.ncol <= TXW + 128) {
@@ -621,21 +627,9 @@ cudaError_t launch_score_t(const T *S, const T *coarse, int H, int W, int k, int
 
 }  // namespace
 
-// Staged row pitch of the grid kernel for a window strip of ncol columns (template width up
-// to 256; wider templates take the generic kernel).
-int score_grid_pitch(int ncol) { return ncol <= TXW + 128 ? TXW + 128 : TXW + 256; }
+// Whether the grid kernel stages a window strip of ncol columns (template width up to 256; wider
+// templates take the generic kernel).
 bool score_grid_fits(int ncol) { return ncol <= TXW + 256; }
-
-size_t score_smem_bytes_for(size_t elem, const BankSpec &bs, const GridSpec &gs, int k)
-{
-    if (gs.G > 0) {
-        const int NR = gs.G + 1;
-        const int NSLOT = gs.G * gs.G + (gs.full ? 1 : 0);
-        return elem * (size_t)NBUF * CH * NR * score_grid_pitch(gs.ncol) + sizeof(int) * ((size_t)NSLOT * k + k + 1) +
-               sizeof(uint64_t) * 2 * NBUF + 16 + 16;
-    }
-    return elem * (size_t)2 * CH * bs.nrow * bs.ncol + sizeof(int) * ((size_t)bs.F * k + 1) + 32;
-}
 
 bool sat_is_u16(int th, int tw) { return (long long)th * tw <= 65535; }
 int sat_pitch(int W) { return (W + 1 + 63) / 64 * 64; }

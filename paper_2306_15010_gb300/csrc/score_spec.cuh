@@ -9,20 +9,15 @@ namespace vqnnf {
 
 constexpr int kMaxFilters = 32;
 constexpr int kMaxRects = 192;
-constexpr int kMaxRows = 2 * kMaxRects;
 
-// One weighted half-open rectangle; ry0 / ry1 index the bank's distinct row offsets.
+// One weighted half-open rectangle.
 struct RectSpec {
     int x0, y0, x1, y1, weight;
-    int ry0, ry1;
 };
 
 // Any bank: F filters, rectangles of filter f are rect[rect_begin[f] .. rect_begin[f+1]).
 struct BankSpec {
     int F;
-    int nrow;                     // distinct row offsets staged per window row
-    int ncol;                     // staged columns per row (256 windows + template width)
-    int roff[kMaxRows];           // the distinct row offsets, ascending
     int rect_begin[kMaxFilters + 1];
     RectSpec rect[kMaxRects];
     float coef[kMaxFilters];      // w_f / A_f
@@ -53,7 +48,6 @@ constexpr int kMaxWGrids = 4;
 constexpr int kMaxWFilters = 5;
 struct WGridSpec {
     int NG;                                   // 0 = not a weighted-grid bank
-    int ncol;
     int nf[kMaxWGrids];
     int bx[kMaxWGrids][4];
     int by[kMaxWGrids][4];
@@ -64,7 +58,6 @@ struct WGridSpec {
     int rowwise[kMaxWGrids][kMaxWFilters];    // sep: 1 = weights by row w[3 r], 0 = weights by column w[c]
 };
 
-size_t score_smem_bytes_for(size_t elem, const BankSpec &bs, const GridSpec &gs, int k);
 // Coarse samples of the integral image, cluster by cluster: S at rows 0, 8, 16, .. and H and at
 // columns 0, 16, 32, .. and the last, element ((row index) * columns + column index) * kp + j,
 // kp = k rounded up to a multiple of 4.  One coalesced read per corner tells for many clusters

@@ -1,6 +1,6 @@
 """Banks that are neither grids nor weighted grids, against the oracle: at the number of warps where the
 kernel goes over to tiles of four rows, with one cluster and every label byte, 16- and 32-bit tables,
-template counts of either sign, and grid banks wider than the grid kernels take."""
+template counts of either sign, many distinct row offsets, and grid banks wider than the grid kernels take."""
 import numpy as np
 import pytest
 import torch
@@ -36,6 +36,7 @@ def _bank(th, tw, F, rects, r):
     (308, 806, 5, 7, 17, 5, 5),          # 25 x 76: one row a warp
     (306, 839, 4, 8, 1, 5, 3),           # the last tile moved up, one cluster
     (60, 75, 33, 31, 256, 6, 20),
+    (270, 300, 260, 253, 9, 5, 7),       # 32-bit table; 68 row offsets
     (41, 300, 40, 20, 130, 6, 4),        # two window rows
     (90, 400, 70, 300, 33, 10, 0),       # a 3 x 3 grid and its full window, too wide for the grid kernels
     (262, 330, 256, 270, 5, 5, 0),       # a 2 x 2 grid, 32-bit table
