@@ -178,31 +178,37 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
 #pragma unroll
         for (int q = 0; q < 8; ++q) red[w][q] = v8[q];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        float tot[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) tot[q] = red[0][q];
+    if (w == 0) {
+        // The tail is latency-bound: each total on a lane of its own (lane 0 the double-float pair of
+        // totals 0 and 1), and every norm's FP64 square root in one evaluation over the lanes.  Ten Lloyd
+        // steps on 64 x 64 pixels, D = 512, k = 64, BF16: 369 us, 384 with one thread for all of it.
+        const int nw = blockDim.x >> 5, mine = min(lane, 7);
+        float tot = red[0][mine], comp = red[0][1];
         for (int u2 = 1; u2 < nw; ++u2) {
             float t, te;
-            two_sum(tot[0], red[u2][0], t, te);
-            tot[0] = t;
-            tot[1] = tot[1] + red[u2][1] + te;
-#pragma unroll
-            for (int q = 2; q < 8; ++q) tot[q] += red[u2][q];
+            two_sum(tot, red[u2][mine], t, te);
+            tot = t;
+            comp = comp + red[u2][1] + te;
         }
         const double u = kU32;
         // ||c*||^2: the compensated sum is within (2u + 2 D u^2) of the exact value (plus the
         // small terms' own rounding, relative u^2 D); n32 rounds it once more
-        const float n32 = __fadd_rn(tot[0], tot[1] + tot[2]);
+        const float n32 = __shfl_sync(0xffffffffu, __fadd_rn(tot, comp + __shfl_sync(0xffffffffu, tot, 2)), 0);
         const double c2 = (double)n32;
         const double en = 4.0 * u * c2 + 1e-37;                 // >= |n32 - ||c*||^2|
         // other norms: sums of D non-negative terms are within gamma_D of the exact value
         const double up = 1.0 + (2.0 * D + 8.0) * u;
         const double margin = 1.0 + 4.0 * u;
-        const double nc = sqrt((c2 + en) * up) * margin;        // ||c*||
-        const double ncc = sqrt((double)tot[3] * up) * margin;  // ||fl32(c*)||
-        const double nd32 = sqrt((double)tot[4] * up) * margin; // ||c* - fl32(c*)||
+        const double root = sqrt(lane == 0 ? (c2 + en) * up : lane == 1 ? (double)D : (double)tot * up);
+        auto root_of = [&](int q) { return __shfl_sync(0xffffffffu, root, q); };
+        const double nc = root_of(0) * margin;                  // ||c*||
+        const double sqrt_D = root_of(1);
+        const double ncc = root_of(3) * margin;                 // ||fl32(c*)||
+        const double nd32 = root_of(4) * margin;                // ||c* - fl32(c*)||
+        const double nhi = root_of(5) * margin;                 // the BF16 planes', and what they leave
+        const double nlo = root_of(6) * margin;
+        const double nd16 = root_of(7) * margin;
+        if (lane != 0) return;
         double a = 0.0, v = 0.0;
         if (prec == VQNNF_PREC_FP32) {
             const double gD = (double)D * u / (1.0 - (double)D * u);
@@ -217,7 +223,7 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
             // rounding of the tensor core are not documented: four times the sequential FP32
             // bound (gacc).  The dot product's error is then at most
             //   X (dc + gacc nq) + ||x' - s_x q_x|| ||c*||,  X >= ||s_x q_x||
-            const double sub = 0.0009765625 * (double)csc * sqrt((double)D) * margin;
+            const double sub = 0.0009765625 * (double)csc * sqrt_D * margin;
             const double dc = 0.0625 * ncc + sub + nd32;
             const double nq = (1.0 + 0.0625) * ncc + sub;
             const double gacc = (double)D * 4.0 * u;
@@ -230,9 +236,6 @@ __global__ void __launch_bounds__(256) prep_centroid_kernel(const float *__restr
             // order and rounding are not documented: take four times the sequential FP32
             // bound.  The x_lo terms (||x_lo|| <= 2^-8 ||x_hi||) are folded into a_j:
             //   |err| <= X [gacc (|hi| + |lo|) + |d|] + X_lo [gacc |hi| + |lo| + |d|] + ...
-            const double nhi = sqrt((double)tot[5] * up) * margin;
-            const double nlo = sqrt((double)tot[6] * up) * margin;
-            const double nd16 = sqrt((double)tot[7] * up) * margin;
             const double gacc = (double)D * 4.0 * u;
             const double a16 = 2.0 * (gacc * (nhi + nlo) + nd16) + 2.0 * 0.00390625 * (gacc * nhi + nlo + nd16);
             if (prec == VQNNF_PREC_FP8) {
