@@ -22,11 +22,31 @@ cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 // ----------------------------------------------------------------------------------
 // Workspace layouts (the same code computes sizes with a null base).
 // ----------------------------------------------------------------------------------
-// Whether an FP8 assignment may take the BF16 second pass.  Below 2^20 feature values its launch and
-// bounds (8 us) cost more than re-scoring, which the chip then does in about one wave: Lloyd steps of a
-// 16 x 19 template, D = 160, take 25 us without it and 33 us with it; from there on re-scoring grows
-// with n D (10 steps, 128 x 128, D = 64: 720 us without it, 428 us with it).
+// Whether an FP8 assignment may take the BF16 second pass.  Its launch costs 2.2 us where it does not
+// run, a sixth of the assignment's kernels or less from 2^20 feature values on (65,536 pixels, D = 64,
+// k = 64: 32 us); where it runs it halves the time and more (10 Lloyd steps, 128 x 128, D = 64, superpixel
+// features: 720 us without it, 428 us).
 bool second_pass_pays(long long n, int D) { return n * D >= (1ll << 20); }
+
+// When it runs, in hundredths of a nanosecond, from timings of both ways (1,024 to 1,048,576 pixels, D = 16
+// to 1,024, k = 16 to 128, 0 to 16 candidates a pixel): re-scoring takes 0.6 ns a pixel and 0.16 ns a
+// candidate while the features stay in registers, 1 ns and 0.9 D / 1000 ns beyond, 1.7 times that while its
+// grid is one block per SM; the pass 6 us, 11 ns per dimension and 0.11 + 0.6 D / 1000 ns a pixel.  Of 480
+// such inputs 14 take the slower way, by 19 % at most.  Counting pixels alone (more than an eighth) chose
+// no fewer, by up to 43 %: 1,024 pixels, D = 1024, two candidates each, 36 us, 23 without the pass.
+SecondPass second_pass(long long n, int D, const FlagList &first, const FlagList &second)
+{
+    const unsigned f = n < 9728 ? 17 : 10;
+    const bool inreg = D <= 512;
+    SecondPass s;
+    s.first = first.count;
+    s.count = second.count;
+    s.left = first.stats + 4;
+    s.per_pixel = f * (inreg ? 6 : 10);
+    s.per_cand = f * (inreg ? 16 : 9 * D / 100) / 10;
+    s.limit = 600000ull + 1100ull * D + (unsigned long long)n * (1100 + 6 * D) / 100;
+    return s;
+}
 
 AssignWs carve_assign(WsCursor &c, long long n, int D, int k, int prec)
 {
@@ -174,10 +194,9 @@ vqnnf_status run_assign(const float *X, long long n, int D, const float *C, int 
         if (e == cudaSuccess) e = record_kernel_event(VQNNF_OP_ASSIGN, 1, s);
     }
     // The FP8 bound (2^-4 relative) leaves most pixels of ordinary features ambiguous, with many
-    // candidates each; re-scoring streams a centroid per candidate from L2.  Above an eighth of the
-    // pixels the BF16 contraction, whose bound leaves 2 %, decides first: it costs one more pass over
-    // the features (1024 x 1024, D = 1024, k = 128, 70 % ambiguous: 0.9 ms, re-scoring all of them
-    // 10.6 ms; an eighth of the pixels at 20 candidates re-score in 1.9 ms, at 8 in 0.8 ms).
+    // candidates each; re-scoring streams a centroid per candidate from L2.  Where that takes longer, the
+    // BF16 contraction, whose bound leaves 2 %, decides first: it costs one more pass over the features
+    // (1024 x 1024, D = 1024, k = 128, 70 % ambiguous: 0.9 ms, re-scoring all of them 10.6 ms).
     SecondPass second = {};
     if (e == cudaSuccess && prec == VQNNF_PREC_FP8 && w.prep.a2 && second_pass_pays(n, D)) {
         CodebookPrep p = w.prep;
@@ -185,7 +204,7 @@ vqnnf_status run_assign(const float *X, long long n, int D, const float *C, int 
         p.v = w.prep.v2;
         FlagList f = w.fl;
         f.count = w.fl.count + 1;
-        second = {w.fl.count, f.count, (unsigned)(n / 8)};
+        second = second_pass(n, D, w.fl, f);
         e = launch_assign_bf16(X, n, D, k, p, labels, f, s, second);
         if (e == cudaErrorNotSupported) {      // a shape the BF16 contraction does not take
             second = {};

@@ -545,8 +545,7 @@ __global__ void __launch_bounds__(256, 2) rescore_kernel(const float *__restrict
     const int lane = threadIdx.x & 31;
     const unsigned wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned nw = (gridDim.x * blockDim.x) >> 5;
-    unsigned listed = *fl.count;
-    if (second.first && listed > second.limit) listed = *second.count;   // the second pass's list
+    const unsigned listed = second.first && second.runs() ? *second.count : *fl.count;   // the second pass's list
     const unsigned n_entries = min(listed, cap);        // the list holds at most cap entries
     const float u = (float)kU32;
     const float rho = ((float)((D + 31) / 32) + 8.0f) * u * 1.01f + 4.0f * u;

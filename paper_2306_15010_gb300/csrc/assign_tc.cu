@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(NT, 1) assign_tc_kernel(const __grid_constant_
                                                           const __grid_constant__ TcArgs g)
 {
     ptx::pdl_enter();
-    if (SECOND && *g.second.first <= g.second.limit) return;   // uniform over the grid
+    if (SECOND && !g.second.runs()) return;                  // uniform over the grid
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int npad = g.npad, D = g.D, nkc = g.nkc, SB = g.sb, SF = g.sf, NB = g.nb, SA = g.sa;

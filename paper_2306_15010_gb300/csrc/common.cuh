@@ -63,12 +63,19 @@ cudaError_t launch_prep_codebook(const float *C, int k, int D, int prec, Codeboo
 cudaError_t launch_assign_fp32(const float *X, long long n, int D, int k,
                                const CodebookPrep &p, uint8_t *labels, FlagList fl,
                                cudaStream_t s);
-// A second pass over pixels that another contraction left ambiguous runs only where that one's
-// count exceeds a limit; its flag list then replaces the first one's (same entries, own counter).
+// A second pass over pixels that another contraction left ambiguous runs only where re-scoring them
+// would take longer, by the number of pixels and of candidates that it left; its flag list then
+// replaces the first one's (same entries, own counter).
 struct SecondPass {
-    const unsigned int *first;    // the first pass's counter (null: not a second pass)
-    const unsigned int *count;    // the second pass's counter
-    unsigned int limit;
+    const unsigned int *first;         // the first pass's counter (null: not a second pass)
+    const unsigned int *count;         // the second pass's counter
+    const unsigned long long *left;    // candidates that the first pass left
+    unsigned int per_pixel, per_cand;  // cost of re-scoring, and what it has to exceed
+    unsigned long long limit;
+    __device__ __forceinline__ bool runs() const
+    {
+        return (unsigned long long)per_pixel * *first + per_cand * *left > limit;
+    }
 };
 cudaError_t launch_assign_bf16(const float *X, long long n, int D, int k,
                                const CodebookPrep &p, uint8_t *labels, FlagList fl,
