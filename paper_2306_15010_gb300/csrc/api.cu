@@ -567,7 +567,7 @@ vqnnf_status vqnnf_score(const uint8_t *q_labels, int H, int W, int k, int th, i
     cudaStream_t s = as_stream(stream);
     WsCursor c{static_cast<char *>(ws), 0};
     ScoreWs sw = carve_score(c, H, W, k, th, tw);
-    cudaError_t e = launch_sat(q_labels, H, W, k, sw.u16, sw.carry, sw.bandsum, sw.S, sw.coarse, s);
+    cudaError_t e = launch_sat(q_labels, H, W, k, sw.u16, sw.carry, sw.bandsum, sw.S, sw.coarse, sw.aux, s);
     if (e != cudaSuccess) return from_cuda(e);
     const int HO = H - th + 1, WO = W - tw + 1;
     return from_cuda(launch_score(sw.S, sw.coarse, sw.u16, H, W, k, HO, WO, bs, gs, wg, t_counts, heatmap, sw.aux,
@@ -645,7 +645,7 @@ vqnnf_status vqnnf_match_host(const float *X_host, int H, int W, int D, const fl
                                 nullptr, w.as, cs);
         }
         const int HO = H - th + 1, WO = W - tw + 1;
-        if (st == VQNNF_OK) st = from_cuda(launch_sat(w.ql, H, W, k, w.sc.u16, w.sc.carry, w.sc.bandsum, w.sc.S, w.sc.coarse, cs));
+        if (st == VQNNF_OK) st = from_cuda(launch_sat(w.ql, H, W, k, w.sc.u16, w.sc.carry, w.sc.bandsum, w.sc.S, w.sc.coarse, w.sc.aux, cs));
         if (st == VQNNF_OK)
             st = from_cuda(launch_score(w.sc.S, w.sc.coarse, w.sc.u16, H, W, k, HO, WO, bs, gs, wg, w.tc, w.heat, w.sc.aux, w.am, cs));
         if (st == VQNNF_OK && heat_host)

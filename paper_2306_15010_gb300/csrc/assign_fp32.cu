@@ -716,7 +716,7 @@ static cudaError_t launch_simt(const float *X, long long n, int D, int k, const 
 {
     using L = SimtTile<TM, TN>;
     const size_t smem = L::smem(k);
-    const cudaError_t e = allow_smem(assign_fp32_kernel<TM, TN, MB>);
+    const cudaError_t e = allow_smem(assign_fp32_kernel<TM, TN, MB>, smem);
     if (e != cudaSuccess) return e;
     const long long blocks = (n + L::BM - 1) / L::BM;
     return launch_pdl(assign_fp32_kernel<TM, TN, MB>, dim3((unsigned)blocks), dim3(NT), smem, s, X, n, D, k, p, labels, fl);

@@ -1226,12 +1226,12 @@ cudaError_t launch_assign_bf16_seg(const float *X, long long n, int D, const Cod
     const long long grid = a.ntiles < sms ? a.ntiles : sms;
     if (nseg == 1) {
         auto kernel = second.first ? assign_tc_kernel<false, false, true> : assign_tc_kernel<false, false>;
-        e = allow_smem(kernel);
+        e = allow_smem(kernel, smem);
         if (e != cudaSuccess) return e;
         e = launch_pdl(kernel, dim3((unsigned)grid), dim3(NT), smem, s, tmA, tmBhi, tmBlo, a);
         if (e != cudaSuccess) return e;
     } else {
-        e = allow_smem(assign_tc_kernel<true, false>);
+        e = allow_smem(assign_tc_kernel<true, false>, smem);
         if (e != cudaSuccess) return e;
         {
         const cudaError_t le_ = launch_pdl(assign_tc_kernel<true, false>, dim3((unsigned)grid), dim3(NT), smem, s, tmA, tmBhi, tmBlo, a);
@@ -1317,7 +1317,7 @@ cudaError_t launch_assign_bf16_stat(const float *X, long long n, int D, const Co
     a.ngroup = ngroup;
     for (int gi = 0; gi <= ngroup; ++gi) a.gs0[gi] = gs0[gi];
     const long long grid = a.ntiles < sms ? a.ntiles : sms;
-    e = allow_smem(assign_tc_kernel<true, true>);
+    e = allow_smem(assign_tc_kernel<true, true>, smem);
     if (e != cudaSuccess) return e;
     {
         const cudaError_t le_ = launch_pdl(assign_tc_kernel<true, true>, dim3((unsigned)grid), dim3(NT), smem, s, tmA, tmBhi, tmBlo, a);
@@ -1393,7 +1393,7 @@ cudaError_t launch_assign_fp8(const float *X, long long n, int D, int k, const C
     a.rs = f8.rs;
     a.labels = labels;
     a.fl = fl;
-    e = allow_smem(assign_fp8_kernel);
+    e = allow_smem(assign_fp8_kernel, smem);
     if (e != cudaSuccess) return e;
     if ((e = record_kernel_event(VQNNF_OP_ASSIGN, 0, s)) != cudaSuccess) return e;
     const long long grid = a.ntiles < sms ? a.ntiles : sms;

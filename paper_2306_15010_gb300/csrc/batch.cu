@@ -574,7 +574,7 @@ vqnnf_status vqnnf_match_batch(const vqnnf_image *q, int nq, const vqnnf_batch_t
             const cudaStream_t ls = nl ? lp->st[l] : s;
             WsCursor sc{w.score_base[l], 0};
             ScoreWs sw = carve_score(sc, q[i].H, q[i].W, t[j].k, t[j].h, t[j].w);
-            e = launch_sat(w.qlab[j], q[i].H, q[i].W, t[j].k, sw.u16, sw.carry, sw.bandsum, sw.S, sw.coarse, ls);
+            e = launch_sat(w.qlab[j], q[i].H, q[i].W, t[j].k, sw.u16, sw.carry, sw.bandsum, sw.S, sw.coarse, sw.aux, ls);
             if (e != cudaSuccess) return from_cuda(e);
             const int HO = q[i].H - t[j].h + 1, WO = q[i].W - t[j].w + 1;
             float *hp = heat ? heat[(size_t)i * nt + j] : w.heat_scratch[l];

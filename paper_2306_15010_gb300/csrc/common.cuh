@@ -124,14 +124,15 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Lifts the kernel's limit on dynamic shared memory to all that a block can have beside `fixed` bytes of
-// static shared memory.  The limit belongs to the function and not to the launch, so every launch sets the
-// same one: one that set its own size could take the room from another host thread between that thread's
-// setting and its launch.
+// For a launch with `bytes` of dynamic shared memory beside `fixed` static ones: lifts the kernel's limit to
+// all that a block can have, where 48 KB do not do.  The limit belongs to the function and not to the
+// launch, so every launch that needs one sets the same: one that set its own size could take the room
+// from another host thread between that thread's setting and its launch.
 constexpr size_t kBlockSmem = 227 * 1024;
 template <typename... KArgs>
-inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t fixed = 0)
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes, size_t fixed = 0)
 {
+    if (bytes + fixed <= 48 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockSmem - fixed));
 }
 

@@ -44,10 +44,15 @@ __device__ int g_score_error = 0;
 constexpr int SW = 64;     // columns per strip (two per lane)
 
 // carry[(y * nS + s) * k + j] = #{x' < 64 s : label(y, x') = j}
+// The first block also clears the score's maximum and probe.
 __global__ void row_carry_kernel(const uint8_t *__restrict__ lab, int W, int k, int nS,
-                                 int *__restrict__ carry)
+                                 int *__restrict__ carry, ScoreAux *aux)
 {
     ptx::pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        aux->amax = 0ull;
+        aux->probe = 0ll;
+    }
     extern __shared__ int hist[];     // [nS][k]
     const int y = blockIdx.x;
     for (int q = threadIdx.x; q < nS * k; q += blockDim.x) hist[q] = 0;
@@ -546,14 +551,14 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
     dim3 grid((WO + TXW - 1) / TXW, HO);
     cudaError_t e;
     if (gs.ncol <= TXW + 128) {
-        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 128>);
+        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 128>, smem);
         if (e != cudaSuccess) return e;
         {
         const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 128>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
         if (le_ != cudaSuccess) return le_;
     }
     } else {
-        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 256>);
+        e = allow_smem(score_grid_kernel<T, G, FULL, TXW + 256>, smem);
         if (e != cudaSuccess) return e;
         {
         const cudaError_t le_ = launch_pdl(score_grid_kernel<T, G, FULL, TXW + 256>, dim3(grid), dim3(STH), smem, s, S, P, k, HO, WO, gs, tc, heat, amax, probe, dense_from);
@@ -565,20 +570,20 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
 
 template <typename T>
 cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, int *bandsum, T *S,
-                         T *coarse, cudaStream_t s)
+                         T *coarse, ScoreAux *aux, cudaStream_t s)
 {
     const int nS = sat_strips(W);
     const int P = sat_pitch(W);
     const int BH = sat_band_rows(H, W, k), nB = sat_bands(H, W, k);
     const size_t hsmem = sizeof(int) * (size_t)nS * k;
-    cudaError_t e = allow_smem(row_carry_kernel);
+    cudaError_t e = allow_smem(row_carry_kernel, hsmem);
     if (e != cudaSuccess) return e;
     {
-        const cudaError_t le_ = launch_pdl(row_carry_kernel, dim3(H), dim3(256), hsmem, s, lab, W, k, nS, carry);
+        const cudaError_t le_ = launch_pdl(row_carry_kernel, dim3(H), dim3(256), hsmem, s, lab, W, k, nS, carry, aux);
         if (le_ != cudaSuccess) return le_;
     }
     const size_t csmem = sizeof(int) * ((size_t)SW * k + k);
-    e = allow_smem(band_sum_kernel);
+    e = allow_smem(band_sum_kernel, csmem);
     if (e != cudaSuccess) return e;
     {
         const cudaError_t le_ = launch_pdl(band_sum_kernel, dim3(dim3(nS, nB)), dim3(256), csmem, s, lab, H, W, k, P, nS, BH, carry, bandsum);
@@ -594,7 +599,7 @@ cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, in
     CUtensorMap map;
     e = make_sat_map(&map, S, sizeof(T) == 2, P, k, H + 1);
     if (e != cudaSuccess) return e;
-    e = allow_smem(sat_write_kernel<T>);
+    e = allow_smem(sat_write_kernel<T>, SatTile<T>::smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(sat_write_kernel<T>, dim3(blocks), dim3(32 * kSatWarps), SatTile<T>::smem, s, map, lab, H, W, k, P, nS, nB,
                    BH, carry, bandsum, coarse);
@@ -664,12 +669,12 @@ int score_ncol(int tw) { return (TXW + tw + 7) / 8 * 8; }
 size_t sat_slack_elems(int tw) { return (size_t)score_ncol(tw) + 64; }
 
 cudaError_t launch_sat(const uint8_t *lab, int H, int W, int k, bool u16, int *carry, int *bandsum,
-                       void *S, void *coarse, cudaStream_t s)
+                       void *S, void *coarse, ScoreAux *aux, cudaStream_t s)
 {
     return u16 ? launch_sat_t<uint16_t>(lab, H, W, k, carry, bandsum, static_cast<uint16_t *>(S),
-                                        static_cast<uint16_t *>(coarse), s)
+                                        static_cast<uint16_t *>(coarse), aux, s)
                : launch_sat_t<uint32_t>(lab, H, W, k, carry, bandsum, static_cast<uint32_t *>(S),
-                                        static_cast<uint32_t *>(coarse), s);
+                                        static_cast<uint32_t *>(coarse), aux, s);
 }
 
 cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, const BankSpec &bs,
@@ -687,9 +692,8 @@ cudaError_t launch_score(const void *S, const void *coarse, bool u16, int H, int
                          const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
                          ScoreAux *aux, int32_t *argmax_yx, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(aux, 0, 16, s);                    // the maximum and the probe
+    cudaError_t e = record_kernel_event(VQNNF_OP_SCORE, 0, s);
     if (e != cudaSuccess) return e;
-    if ((e = record_kernel_event(VQNNF_OP_SCORE, 0, s)) != cudaSuccess) return e;
     e = u16 ? launch_score_t(static_cast<const uint16_t *>(S), static_cast<const uint16_t *>(coarse), H, W, k, HO, WO, bs,
                              gs, ws, tc, heat, aux, s)
             : launch_score_t(static_cast<const uint32_t *>(S), static_cast<const uint32_t *>(coarse), H, W, k, HO, WO, bs,

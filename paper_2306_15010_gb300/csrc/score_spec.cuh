@@ -78,12 +78,8 @@ cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int ro
 int score_ncol(int tw);
 bool score_grid_fits(int ncol);   // the grid kernel stages at most TXW + 256 columns
 size_t sat_slack_elems(int tw);
-cudaError_t launch_sat(const uint8_t *lab, int H, int W, int k, bool u16, int *carry, int *bandsum,
-                       void *S, void *coarse, cudaStream_t s);
-cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, const BankSpec &bs,
-                                    int32_t *counts, cudaStream_t s);
-// Device words of one score: the maximum's key and the probe (both start at zero), and the grid
-// bank's template side.
+// Device words of one score: the maximum's key and the probe (both zero after launch_sat), and
+// the grid bank's template side.
 constexpr int kMaxSlots = 17;
 struct ScoreAux {
     unsigned long long amax;
@@ -91,6 +87,10 @@ struct ScoreAux {
     int tsum[kMaxSlots];                          // per slot: sum of the positive template counts
     alignas(16) int t[kMaxSlots][256];            // the slots' template counts
 };
+cudaError_t launch_sat(const uint8_t *lab, int H, int W, int k, bool u16, int *carry, int *bandsum,
+                       void *S, void *coarse, ScoreAux *aux, cudaStream_t s);
+cudaError_t launch_filter_responses(const uint8_t *lab, int h, int w, int k, const BankSpec &bs,
+                                    int32_t *counts, cudaStream_t s);
 cudaError_t launch_score(const void *S, const void *coarse, bool u16, int H, int W, int k, int HO, int WO,
                          const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,
                          ScoreAux *aux, int32_t *argmax_yx, cudaStream_t s);

@@ -977,7 +977,7 @@ cudaError_t launch_soft_p_ki(const float *X, long long n, long long npi, int D, 
     constexpr int PTK = SoftTile<KI>::PT;
     const size_t sm = sizeof(float) * SoftStage<KI>::floats(k);
     const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(C)) % 16 == 0;
-    cudaError_t e = allow_smem(soft_p_kernel<KI>);
+    cudaError_t e = allow_smem(soft_p_kernel<KI>, sm);
     if (e != cudaSuccess) return e;
     soft_p_kernel<KI><<<(unsigned)((n + PTK - 1) / PTK), 256, sm, s>>>(X, n, npi, D, C, k, tau, vec, P);
     return cudaGetLastError();
@@ -996,7 +996,7 @@ cudaError_t launch_soft_back_ki(const float *X, long long n, long long npi, int 
                                 float tau, const float *P, const float *Gp, float *A, float *dX, cudaStream_t s)
 {
     const size_t sm = sizeof(float) * ((PT + 16 * KI) * (DCH + 1) + 2 * PT * (16 * KI + 1) + PT + 16 * KI * (PT + 4));
-    cudaError_t e = allow_smem(soft_back_kernel<KI>);
+    cudaError_t e = allow_smem(soft_back_kernel<KI>, sm);
     if (e != cudaSuccess) return e;
     soft_back_kernel<KI><<<(unsigned)((n + PT - 1) / PT), 256, sm, s>>>(X, n, npi, D, C, k, tau, P, Gp, A, dX);
     return cudaGetLastError();
@@ -1024,7 +1024,7 @@ BoxSpec box_spec(const SoftGrid &sg)
 template <int NW, int NH>
 cudaError_t launch_box(SoftWs &w, int B, int H, int W, int k, const SoftGrid &sg, const BoxSpec &bs, size_t smem, cudaStream_t s)
 {
-    const cudaError_t e = allow_smem(box_kernel<NW, NH>);
+    const cudaError_t e = allow_smem(box_kernel<NW, NH>, smem);
     if (e != cudaSuccess) return e;
     box_kernel<NW, NH><<<dim3((W - bs.wlo + BXT) / BXT, (H - bs.hlo + BYT) / BYT, (unsigned)(B * k)), 256, smem, s>>>(
         w.P, H, W, k, sg.ns, bs, w.BX);
@@ -1037,7 +1037,7 @@ cudaError_t launch_gather_j(const SoftWs &w, const float *dheat, const float *wf
 {
     const int h = sg.hgt[sg.size_h[is]];
     const size_t zs = sizeof(float) * J * GR * gather_pitch(W);   // up to ~198 KB
-    cudaError_t e = allow_smem(soft_gather_kernel<MC, J>, 2048);
+    cudaError_t e = allow_smem(soft_gather_kernel<MC, J>, zs, 2048);
     if (e != cudaSuccess) return e;
     const long long nblk = (long long)B * ((k + J - 1) / J) * ((H - h + GR) / GR);
     soft_gather_kernel<MC, J><<<(unsigned)nblk, 256, zs, s>>>(w.BX, dheat, w.T, wf, H, W, k, HO, WO, sg, is,
@@ -1146,7 +1146,7 @@ cudaError_t soft_forward(const float *Qf, int B, int H, int W, const float *Tf, 
     for (int iw = 0; iw < sg.nw && !fused; ++iw) {
         const int wd = sg.wid[iw];
         const size_t rs = row_box_smem(wd);                   // up to ~56 KB (W <= 12288)
-        e = allow_smem(row_box_kernel);
+        e = allow_smem(row_box_kernel, rs);
         if (e != cudaSuccess) return e;
         dim3 g((unsigned)(planes * H), (W - wd + RBX) / RBX);
         row_box_kernel<<<g, 128, rs, s>>>(w.P, W, wd, w.RW + (size_t)iw * planes * H * W);
@@ -1196,7 +1196,7 @@ cudaError_t soft_backward(const float *Qf, int B, int H, int W, const float *Tf,
     for (int is = 0; is < sg.ns; ++is) hmax = ac.h[is] > hmax ? ac.h[is] : hmax;
     const size_t csm = adj_smem(hmax);
     if (csm <= kTileSmem) {
-        e = allow_smem(adj_tile_kernel);
+        e = allow_smem(adj_tile_kernel, csm);
         if (e != cudaSuccess) return e;
         adj_tile_kernel<<<dim3((W + BXT - 1) / BXT, (H + BYT - 1) / BYT, (unsigned)planes), 256, csm, s>>>(
             w.R2, planes * H * W, H, W, ac, hmax, W % 4 == 0, w.G);

@@ -373,7 +373,7 @@ template <int KP>
 cudaError_t launch_kp(const SoftTcArgs &a, int grid, cudaStream_t s)
 {
     const int sm = smem_bytes_for(KP, a.nd);
-    cudaError_t e = allow_smem(soft_grad_tc_kernel<KP>);
+    cudaError_t e = allow_smem(soft_grad_tc_kernel<KP>, sm);
     if (e != cudaSuccess) return e;
     soft_grad_tc_kernel<KP><<<grid, UNT, sm, s>>>(a);
     return cudaGetLastError();
