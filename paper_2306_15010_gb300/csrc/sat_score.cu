@@ -515,6 +515,148 @@ __global__ void __launch_bounds__(STH, G <= 3 ? 8 : 6) score_grid_kernel(const T
     }
 }
 
+// Weighted-grid bank (WGridSpec) over a 32-bit table, where a probe finds it cheaper than the tiles
+// (wgrid_probe_kernel): grid by grid, one pass over the clusters stages that grid's four corner rows;
+// per cluster and window the 16 corners give the 9 cell counts, each of the grid's filters is their
+// integer weighting R, and |t - R| is summed exactly per filter.  The weights and coefficients are
+// kernel parameters indexed at compile time.  After each grid's pass its filters' sums enter the
+// float heatmap accumulator (fixed order).
+// Bound by the shared-memory loads, 16 a window and cluster; a window takes 24 bytes a pair from L2, its
+// columns shared by the block's 512 windows, where a tile takes 72.  1024 x 1024, k = 64, 300 x 256
+// template, every cluster in every window, one filter per grid: 0.56 ms, the tiles 0.97.
+template <int NG, int NCOLP>
+__global__ void __launch_bounds__(STH, 6) score_wgrid_kernel(const uint32_t *__restrict__ S, int P, int k,
+                                                          int HO, int WO, int ncol, WGridSpec ws,
+                                                          const int32_t *__restrict__ tcounts,
+                                                          float *__restrict__ heat,
+                                                          unsigned long long *amax, const long long *probe)
+{
+    ptx::pdl_enter();
+    if (*probe <= 0) return;                                   // the tile kernel takes this image
+    using T = uint32_t;
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    constexpr int chunk_elems = 4 * NCOLP;                    // one cluster, four corner rows
+    T *bufs = reinterpret_cast<T *>(smem_raw);                 // [NBUF][chunk]
+    int *tc = reinterpret_cast<int *>(bufs + NBUF * chunk_elems);   // [NG][5][k]
+    uint64_t *full = reinterpret_cast<uint64_t *>(tc + NG * kMaxWFilters * k + ((NG * kMaxWFilters * k) & 1));
+    uint64_t *empty = full + NBUF;
+    int *n_issued = reinterpret_cast<int *>(empty + NBUF);
+    const int y = blockIdx.y;
+    const int x0 = blockIdx.x * TXW;
+    const int lane = threadIdx.x & 31;
+    const int nchunk = NG * k;                                 // chunk ci: grid ci / k, cluster ci % k
+    for (int q = threadIdx.x; q < NG * kMaxWFilters * k; q += blockDim.x) {
+        const int gf = q / k, j = q % k, g = gf / kMaxWFilters, f = gf % kMaxWFilters;
+        tc[q] = f < ws.nf[g] ? tcounts[(size_t)ws.filt[g][f] * k + j] : 0;
+    }
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < NBUF; ++b) {
+            ptx::mbar_init(&full[b], 1);
+            ptx::mbar_init(&empty[b], STH / 32);
+        }
+        ptx::fence_barrier_init();
+        int c = 0;
+        for (; c < NBUF - 1 && c < nchunk; ++c)
+            issue_chunk<T>(bufs + c * chunk_elems, S, k, P, y, x0, c % k, ncol, NCOLP, ws.by[c / k], 4, &full[c]);
+        *n_issued = c;
+    }
+    __syncthreads();
+    float hs[WPT];
+#pragma unroll
+    for (int w = 0; w < WPT; ++w) hs[w] = 0.f;
+    bool ok = true;
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        const int nf = ws.nf[g];
+        int acc[WPT][kMaxWFilters];
+#pragma unroll
+        for (int w = 0; w < WPT; ++w)
+#pragma unroll
+            for (int f = 0; f < kMaxWFilters; ++f) acc[w][f] = 0;
+        int off[4];
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) off[cc] = ws.bx[g][cc];
+        for (int j = 0; ok && j < k; ++j) {
+            const int ch = g * k + j;
+            const int b = ch % NBUF;
+            if (threadIdx.x == 0 && ch + NBUF - 1 < nchunk) {
+                const int nb = (ch + NBUF - 1) % NBUF;
+                const int use = (ch + NBUF - 1) / NBUF;
+                if (use > 0)
+                    ok = ptx::mbar_wait_bounded(&empty[nb], (use - 1) & 1, &g_score_error, (int)VQNNF_ETIMEOUT);
+                if (ok) {
+                    const int cn = ch + NBUF - 1;
+                    issue_chunk<T>(bufs + nb * chunk_elems, S, k, P, y, x0, cn % k, ncol, NCOLP, ws.by[cn / k], 4,
+                                   &full[nb]);
+                    *n_issued = cn + 1;
+                }
+            }
+            ok = __all_sync(0xffffffffu, ok && ptx::mbar_wait_bounded(&full[b], (ch / NBUF) & 1, &g_score_error,
+                                                                      (int)VQNNF_ETIMEOUT));
+            if (!ok) break;
+            const T *cur = bufs + b * chunk_elems + threadIdx.x;
+            int t[kMaxWFilters];
+#pragma unroll
+            for (int f = 0; f < kMaxWFilters; ++f) t[f] = tc[(g * kMaxWFilters + f) * k + j];
+#pragma unroll
+            for (int w = 0; w < WPT; ++w) {
+                int cr[4][4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) cr[r][cc] = (int)cur[off[cc] + r * NCOLP + w * STH];
+                int n[9];
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+#pragma unroll
+                    for (int cc = 0; cc < 3; ++cc)
+                        n[r * 3 + cc] = box<T>(cr[r + 1][cc + 1], cr[r + 1][cc], cr[r][cc + 1], cr[r][cc]);
+#pragma unroll
+                for (int f = 0; f < kMaxWFilters; ++f) {
+                    if (f >= nf) break;
+                    int R = 0;
+#pragma unroll
+                    for (int c = 0; c < 9; ++c) R += ws.w[g][f][c] * n[c];
+                    acc[w][f] += abs(t[f] - R);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(&empty[b]))
+                                        : "memory");
+        }
+#pragma unroll
+        for (int f = 0; f < kMaxWFilters; ++f) {
+            if (f >= nf) break;
+#pragma unroll
+            for (int w = 0; w < WPT; ++w) hs[w] = fmaf(ws.coef[g][f], (float)acc[w][f], hs[w]);
+        }
+    }
+    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
+        const int issued = *n_issued;
+        for (int c = max(0, issued - NBUF); c < issued; ++c)
+            ptx::mbar_wait_bounded(&full[c % NBUF], (c / NBUF) & 1, &g_score_error, (int)VQNNF_ETIMEOUT);
+    }
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int w = 0; w < WPT; ++w) {
+        const int x = x0 + threadIdx.x + w * STH;
+        const float h = -hs[w];
+        if (ok && x < WO) {
+            heat[(size_t)y * WO + x] = h;
+            const unsigned long long key = pack_key(h, (unsigned)(y * WO + x));
+            best = key > best ? key : best;
+        }
+    }
+    if (amax) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+            best = other > best ? other : best;
+        }
+        if ((threadIdx.x & 31) == 0 && best) atomicMax(amax, best);
+    }
+}
+
 // Self-test of the bounded waits: one thread waits on an mbarrier that nothing completes.  No
 // copy is issued, so nothing is in flight when the wait gives up after `limit` SM cycles and
 // records VQNNF_ETIMEOUT in the score kernels' error word.
@@ -568,6 +710,23 @@ cudaError_t launch_grid(const T *S, int P, int k, int HO, int WO, const GridSpec
     return cudaGetLastError();
 }
 
+template <int NG>
+cudaError_t launch_wgrid_dense(const uint32_t *S, int P, int k, int HO, int WO, const WGridSpec &ws, const int32_t *tc, float *heat,
+                               ScoreAux *aux, cudaStream_t s)
+{
+    int w = 0;
+    for (int g = 0; g < NG; ++g) w = ws.bx[g][3] > w ? ws.bx[g][3] : w;
+    const int ncol = score_ncol(w);
+    const bool narrow = ncol <= TXW + 128;
+    const size_t smem = sizeof(uint32_t) * (size_t)NBUF * 4 * (narrow ? TXW + 128 : TXW + 256) +
+                        sizeof(int) * ((size_t)NG * kMaxWFilters * k + 1) + sizeof(uint64_t) * 2 * NBUF + 16 + 16;
+    auto kernel = narrow ? score_wgrid_kernel<NG, TXW + 128> : score_wgrid_kernel<NG, TXW + 256>;
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3((WO + TXW - 1) / TXW, HO), dim3(STH), smem, s, S, P, k, HO, WO, ncol, ws, tc, heat, &aux->amax,
+                      &aux->probe);
+}
+
 template <typename T>
 cudaError_t launch_sat_t(const uint8_t *lab, int H, int W, int k, int *carry, int *bandsum, T *S,
                          T *coarse, ScoreAux *aux, cudaStream_t s)
@@ -614,8 +773,20 @@ cudaError_t launch_score_t(const T *S, const T *coarse, int H, int W, int k, int
 {
     const int P = sat_pitch(W);
     long long dense_from = 0;
-    const ScoreRoute route = gs.G == 0 ? kScoreTiles : score_grid_route(HO, WO, k, P, gs.by[gs.G]);
     cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(T) == 4)
+        if (gs.G == 0 && score_wgrid_probed(ws, k, P, HO)) {
+            e = launch_wgrid_probe(coarse, W, k, HO, WO, ws, aux, s);
+            if (e == cudaSuccess) e = launch_score_tiles(S, coarse, false, W, k, HO, WO, bs, gs, ws, tc, heat, aux, 0, s);
+            if (e != cudaSuccess) return e;
+            switch (ws.NG) {
+            case 1: return launch_wgrid_dense<1>(S, P, k, HO, WO, ws, tc, heat, aux, s);
+            case 2: return launch_wgrid_dense<2>(S, P, k, HO, WO, ws, tc, heat, aux, s);
+            case 3: return launch_wgrid_dense<3>(S, P, k, HO, WO, ws, tc, heat, aux, s);
+            default: return launch_wgrid_dense<4>(S, P, k, HO, WO, ws, tc, heat, aux, s);
+            }
+        }
+    const ScoreRoute route = gs.G == 0 ? kScoreTiles : score_grid_route(HO, WO, k, P, gs.by[gs.G]);
     if (route == kScoreProbe) e = launch_score_probe(coarse, sizeof(T) == 2, W, k, HO, WO, gs, tc, aux, &dense_from, s);
     if (e == cudaSuccess && route != kScoreDense)
         e = launch_score_tiles(S, coarse, sizeof(T) == 2, W, k, HO, WO, bs, gs, ws, tc, heat, aux, dense_from, s);

@@ -100,6 +100,10 @@ enum ScoreRoute { kScoreTiles, kScoreDense, kScoreProbe };
 ScoreRoute score_grid_route(int HO, int WO, int k, int P, int th);
 cudaError_t launch_score_probe(const void *coarse, bool u16, int W, int k, int HO, int WO, const GridSpec &gs,
                                const int32_t *tc, ScoreAux *aux, long long *dense_from, cudaStream_t s);
+// Whether a weighted grid over a 32-bit table is probed, and the probe: aux->probe > 0 where the dense
+// kernel is cheaper (launch_score_tiles then returns at once on the device).
+bool score_wgrid_probed(const WGridSpec &ws, int k, int P, int HO);
+cudaError_t launch_wgrid_probe(const void *coarse, int W, int k, int HO, int WO, const WGridSpec &ws, ScoreAux *aux, cudaStream_t s);
 // A grid bank only where aux->probe <= dense_from, after the probe.
 cudaError_t launch_score_tiles(const void *S, const void *coarse, bool u16, int W, int k, int HO, int WO,
                                const BankSpec &bs, const GridSpec &gs, const WGridSpec &ws, const int32_t *tc, float *heat,

@@ -376,11 +376,13 @@ struct WTile {
 template <typename T, bool SEP>
 __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, int HO, int WO, WGridSpec ws, unsigned test,
                                                                    const int32_t *__restrict__ tcounts,
-                                                                   float *__restrict__ heat, unsigned long long *amax)
+                                                                   float *__restrict__ heat, unsigned long long *amax,
+                                                                   const long long *probe)
 {
     using L = WTile<T, SEP>;
     constexpr int E = L::E, TY = kWY;
     ptx::pdl_enter();
+    if (sizeof(T) == 4 && probe && *probe > 0) return;       // the dense kernel takes this image
     __shared__ __align__(16) uint8_t stage_s[TW][WNST][L::STAGE];
     __shared__ uint16_t list_s[TW][kMaxWGrids * kMaxK];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
@@ -692,6 +694,32 @@ __global__ void __launch_bounds__(128) score_probe_kernel(Sat<T> sat, int HO, in
     }
 }
 
+// The same for a weighted grid over a 32-bit table: one warp per sampled 32 x 4 tile and grid.  With
+// every cluster visited a pair costs a tile 0.80 to 1.35 ns, and the dense kernel 0.51 to 0.67 ns and 0.09 to
+// 0.10 for every further filter of the grid (1024 x 1024 to 2048 x 2048, templates of 300 x 256 to 800 x
+// 100, 1 to 5 filters a grid); `dense` has the latter, in hundredths of a nanosecond, per grid.
+constexpr int kWTileCost = 110;    // of a pair that a tile visits
+struct WGridCost {
+    int dense[kMaxWGrids];
+};
+__global__ void __launch_bounds__(128) wgrid_probe_kernel(Sat<uint32_t> sat, int HO, int WO, int ntx, int nsample, int step, WGridSpec ws,
+                                                          WGridCost cost, ScoreAux *aux)
+{
+    ptx::pdl_enter();
+    const int lane = threadIdx.x & 31, k = sat.k;
+    const int id = blockIdx.x * 4 + (threadIdx.x >> 5), g = id % ws.NG, i = id / ws.NG;
+    if (i >= nsample) return;
+    const long long tile = (long long)i * step;
+    const int X0 = (int)(tile % ntx) * 32, rows = min(4, HO), Y0 = min((int)(tile / ntx) * 4, HO - rows), xe = min(X0 + 31, WO - 1);
+    const Region<uint32_t> reg(sat, X0 + ws.bx[g][0], Y0 + ws.by[g][0], xe + ws.bx[g][3], Y0 + rows - 1 + ws.by[g][3]);
+    int visited = 0;
+    for (int j = 4 * lane; j < k; j += 128) visited += __popc(reg.holds4(j) & (k - j >= 4 ? 15u : (1u << (k - j)) - 1u));
+    visited = __reduce_add_sync(0xffffffffu, visited);
+    if (lane == 0)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&aux->probe),
+                  (unsigned long long)(long long)(kWTileCost * visited - cost.dense[g] * k));
+}
+
 // Slots whose region, swept over a tile of w x h windows, is tested.
 template <typename T>
 unsigned slot_tests(const GridSpec &gs, int w, int h)
@@ -716,18 +744,24 @@ bool wgrid_fits(const WGridSpec &ws, int k, int plane16)
 }
 
 template <typename T>
-cudaError_t launch_wgrid(const Sat<T> &sat, int HO, int WO, const WGridSpec &ws, const int32_t *tc, float *heat,
-                         unsigned long long *amax, cudaStream_t s)
+unsigned wgrid_tests(const WGridSpec &ws)
 {
     unsigned test = 0;
-    bool sep = true;
-    for (int g = 0; g < ws.NG; ++g) {
-        sep = sep && ws.sep[g];
+    for (int g = 0; g < ws.NG; ++g)
         test |= (unsigned)testable<T>(ws.bx[g][3] - ws.bx[g][0] + 31, ws.by[g][3] - ws.by[g][0] + kWY - 1) << g;
-    }
+    return test;
+}
+
+template <typename T>
+cudaError_t launch_wgrid(const Sat<T> &sat, int HO, int WO, const WGridSpec &ws, const int32_t *tc, float *heat,
+                         ScoreAux *aux, cudaStream_t s)
+{
+    bool sep = true;
+    for (int g = 0; g < ws.NG; ++g) sep = sep && ws.sep[g];
+    const long long *probe = sizeof(T) == 4 && score_wgrid_probed(ws, sat.k, sat.P, HO) ? &aux->probe : nullptr;
     return launch_pdl(sep ? score_wgrid_tile_kernel<T, true> : score_wgrid_tile_kernel<T, false>,
-                      dim3((WO + 32 * TW - 1) / (32 * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), 0, s, sat, HO, WO, ws, test, tc,
-                      heat, amax);
+                      dim3((WO + 32 * TW - 1) / (32 * TW), (HO + kWY - 1) / kWY), dim3(32 * TW), 0, s, sat, HO, WO, ws,
+                      wgrid_tests<T>(ws), tc, heat, &aux->amax, probe);
 }
 
 template <typename T>
@@ -745,7 +779,7 @@ cudaError_t launch_tiles_t(const Sat<T> &sat, int HO, int WO, const BankSpec &bs
     if (gs.G > 0)
         return launch_pdl(score_grid_tile_kernel<T, 2, kGridY>, dim3((WO + 64 * TW - 1) / (64 * TW), (HO + kGridY - 1) / kGridY), dim3(32 * TW),
                           0, s, sat, HO, WO, gs, slot_tests<T>(gs, 64, kGridY), heat, aux, dense_from);
-    if (wgrid_fits(ws, sat.k, sat.P / WTile<T, true>::E)) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, amax, s);
+    if (wgrid_fits(ws, sat.k, sat.P / WTile<T, true>::E)) return launch_wgrid<T>(sat, HO, WO, ws, tc, heat, aux, s);
     if (HO >= 4 && (long long)((WO + 31) / 32) * ((HO + 3) / 4) >= kGenericWarps)
         return launch_pdl(score_generic_kernel<T, 4>, dim3((WO + 32 * TW - 1) / (32 * TW), (HO + 3) / 4), dim3(32 * TW), 0, s,
                           sat, HO, WO, bs, tc, heat, amax);
@@ -764,6 +798,35 @@ ScoreRoute score_grid_route(int HO, int WO, int k, int P, int th)
     const long long tiles = (long long)((WO + 63) / 64) * ((HO + 3) / 4);
     const bool far = (long long)(th + 4) * k * (P / 4) >= (1ll << 32);
     return HO < 4 || k <= 16 || tiles < 512 || far ? kScoreDense : kScoreProbe;
+}
+
+// Where every filter weights whole rows or columns, three or more of them a grid, the tiles are the faster
+// with every cluster visited too (300 x 256 template, 1024 x 1024, k = 64, five filters: 0.81 against 0.91
+// ms), and there is no probe (3 us, and 3 for the kernel that returns).  The dense grid has a row of blocks
+// per window row.
+bool score_wgrid_probed(const WGridSpec &ws, int k, int P, int HO)
+{
+    int F = 0;
+    bool sep = true;
+    for (int g = 0; g < ws.NG; ++g) {
+        F += ws.nf[g];
+        sep = sep && ws.sep[g];
+    }
+    return wgrid_fits(ws, k, P / WTile<uint32_t, true>::E) && HO <= 65535 && !(sep && F >= 3 * ws.NG);
+}
+
+cudaError_t launch_wgrid_probe(const void *coarse, int W, int k, int HO, int WO, const WGridSpec &ws, ScoreAux *aux, cudaStream_t s)
+{
+    const int ntx = (WO + 31) / 32;
+    const long long ntile = (long long)ntx * ((HO + 3) / 4);
+    const int step = (int)(ntile / 509 > 1 ? (ntile / 509) | 1 : 1);      // about 500 tiles
+    const int n = (int)((ntile + step - 1) / step);
+    // below two blocks per SM of 512 windows each the dense kernel has too few in flight
+    const bool few = (long long)HO * ((WO + 511) / 512) < 304;
+    WGridCost cost;
+    for (int g = 0; g < kMaxWGrids; ++g) cost.dense[g] = (45 + 10 * ws.nf[g]) * (few ? 16 : 10) / 10;
+    return launch_pdl(wgrid_probe_kernel, dim3((unsigned)((n * ws.NG + 3) / 4)), dim3(128), 0, s,
+                      make_sat<uint32_t>(nullptr, coarse, W, k), HO, WO, ntx, n, step, ws, cost, aux);
 }
 
 cudaError_t launch_score_probe(const void *coarse, bool u16, int W, int k, int HO, int WO, const GridSpec &gs,
