@@ -14,7 +14,9 @@
 //
 // What bounds it: instruction issue and the corner rows' way from L2 into shared memory, in that
 // order (ncu, 2048 x 2048: 70 % and 60 % of peak before the pair list, 2.3 KB per pair and tile).
-// Tiles of 64 x 4 windows with three staged pairs and 14 blocks per SM take 0.45 ms there; 64 x 8
+// Tiles of 64 x 4 windows with three staged pairs take 0.43 ms there, 12 blocks to an SM (18.9 KB of
+// shared memory each, 80 registers); with 72 registers, and 20 bytes of spills, for 14 blocks that
+// shared memory does not hold 0.45, with 96 for 10 blocks 0.46 ms.  64 x 8
 // took 0.46 to 0.51, 128 x 4 0.52, 32 x 4 0.54 ms, two staged pairs 0.49 ms, loads from global memory
 // straight into registers 0.48 ms and more, a table laid out by 64-column strips the same.  The
 // dense kernel (sat_score.cu: every cluster, staged for 512 windows) takes 1.13 ms.  Testing against
@@ -193,7 +195,7 @@ constexpr int kPairs = 512;        // a warp's list: at least the pairs of four 
 
 // `test`: the slots whose region is tested.
 template <typename T, int NX, int TY>
-__global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 14 : 1) score_grid_tile_kernel(Sat<T> sat, int HO, int WO, GridSpec gs, unsigned test,
+__global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 12 : 1) score_grid_tile_kernel(Sat<T> sat, int HO, int WO, GridSpec gs, unsigned test,
                                                                   float *__restrict__ heat, ScoreAux *aux,
                                                                   long long dense_from)
 {
