@@ -1021,6 +1021,15 @@ BoxSpec box_spec(const SoftGrid &sg)
     return bs;
 }
 
+// Whether the box sums take one kernel: cells up to about 60 a side, where two blocks of the tile's shared
+// memory fit an SM.  There (cells of 58 and 59, a training step of 2 x 512 x 512, k = 64) both ways take
+// 1.30 ms.
+bool boxes_fused(const SoftGrid &sg)
+{
+    const BoxSpec bx = box_spec(sg);
+    return box_smem(sg.nw, bx.wlo, bx.hlo) <= kTileSmem;
+}
+
 template <int NW, int NH>
 cudaError_t launch_box(SoftWs &w, int B, int H, int W, int k, const SoftGrid &sg, const BoxSpec &bs, size_t smem, cudaStream_t s)
 {
@@ -1108,7 +1117,7 @@ SoftWs carve_soft(WsCursor &c, int B, int H, int W, int D, int k, int th, int tw
     SoftWs w;
     const size_t plane = (size_t)H * W;
     w.P = c.take<float>((size_t)B * k * plane);
-    w.RW = c.take<float>((size_t)B * sg.nw * k * plane);
+    w.RW = boxes_fused(sg) ? nullptr : c.take<float>((size_t)B * sg.nw * k * plane);
     w.BX = c.take<float>((size_t)B * sg.ns * k * plane);
     w.Pt = c.take<float>((size_t)k * th * tw);
     w.T = c.take<float>((size_t)sg.F * k);
@@ -1135,9 +1144,7 @@ cudaError_t soft_forward(const float *Qf, int B, int H, int W, const float *Tf, 
     const long long planes = (long long)B * k;
     const BoxSpec bx = box_spec(sg);
     const size_t bsm = box_smem(sg.nw, bx.wlo, bx.hlo);
-    // Cells up to about 60 a side: two blocks of the tile's shared memory fit an SM.  There (cells of
-    // 58 and 59, a training step of 2 x 512 x 512, k = 64) both ways take 1.30 ms.
-    const bool fused = bsm <= kTileSmem;
+    const bool fused = boxes_fused(sg);
     if (fused) {
         e = sg.nw == 1 ? (sg.nh == 1 ? launch_box<1, 1>(w, B, H, W, k, sg, bx, bsm, s) : launch_box<1, 2>(w, B, H, W, k, sg, bx, bsm, s))
                        : (sg.nh == 1 ? launch_box<2, 1>(w, B, H, W, k, sg, bx, bsm, s) : launch_box<2, 2>(w, B, H, W, k, sg, bx, bsm, s));

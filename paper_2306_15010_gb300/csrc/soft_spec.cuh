@@ -28,7 +28,7 @@ struct SoftGrid {
 
 struct SoftWs {
     float *P;      // B x k x H x W     query soft assignment (planar), kept for the backward
-    float *RW;     // nw x B x k x H x W row sums of each cell width
+    float *RW;     // nw x B x k x H x W row sums of each cell width (null where one kernel takes the box sums)
     float *BX;     // B x ns x k x H x W box sums of each cell size (the query soft counts)
     float *Pt;     // k x th x tw       template soft assignment, kept for the backward
     float *T;      // F x k             template soft counts

@@ -32,3 +32,16 @@ def test_smaller_query_never_needs_more():
         h, w, kk = _smaller(r, H, W, k, th, tw)
         assert score(h, w, kk, th, tw) <= score(H, W, k, th, tw), (H, W, k, h, w, kk, th, tw)
         assert host(h, w, min(kk, th * tw), th, tw) <= host(H, W, min(k, th * tw), th, tw), (H, W, k, h, w, kk, th, tw)
+
+
+def test_soft_workspace_holds_no_row_sums_where_one_kernel_takes_the_boxes():
+    B, H, W, D, k, side, G = 8, 512, 512, 256, 64, 64, 3
+    from paper_2306_15010_gb300 import soft
+    plane = 4 * B * k * H * W
+    classes = 4                                          # cells of 21 and 22 pixels either way
+    used = plane * (1 + 2 * classes + 2)                 # p, box sums and adjoint rows by class, two gradients
+    l1 = 4 * B * G * G * (H - side + 1) ** 2
+    got = soft.soft_workspace_bytes(B, H, W, D, k, side, side, G)
+    assert used + l1 <= got < used + l1 + plane // 2
+    # cells too large for it keep them
+    assert soft.soft_workspace_bytes(1, 300, 300, 4, 8, 200, 200, 1) >= 4 * 8 * 300 * 300 * (1 + 1 + 2 + 2)
