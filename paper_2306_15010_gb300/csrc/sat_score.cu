@@ -339,21 +339,6 @@ constexpr int TXW = STH * WPT;    // windows per block along x
 constexpr int CH = 1;             // clusters per staged chunk
 constexpr int NBUF = 4;           // staging buffers of the grid kernel
 
-__device__ __forceinline__ unsigned long long pack_key(float v, unsigned idx)
-{
-    unsigned b = __float_as_uint(v);
-    b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // order-preserving
-    return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - idx);
-}
-
-// Box count from four integral-image values; exact mod 2^16 for the 16-bit table.
-template <typename T>
-__device__ __forceinline__ int box(int s11, int s10, int s01, int s00)
-{
-    const int v = s11 - s10 - s01 + s00;
-    return sizeof(T) == 2 ? (v & 0xFFFF) : v;
-}
-
 // Thread 0 issues the bulk copies of one chunk of corner rows: for cluster c of the chunk
 // and corner row rr, the ncol elements of S starting at column x0, staged pitch elements apart.
 template <typename T>

@@ -78,6 +78,22 @@ cudaError_t make_sat_map(CUtensorMap *m, void *S, bool u16, int P, int k, int ro
 int score_ncol(int tw);
 bool score_grid_fits(int ncol);   // the grid kernel stages at most TXW + 256 columns
 size_t sat_slack_elems(int tw);
+
+// The maximum's key: larger for the larger value, then for the lower window index.
+__device__ __forceinline__ unsigned long long pack_key(float v, unsigned idx)
+{
+    unsigned b = __float_as_uint(v);
+    b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // order-preserving
+    return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - idx);
+}
+// Box count from four integral-image values; exact mod 2^16 for the 16-bit table.
+template <typename T>
+__device__ __forceinline__ int box(int s11, int s10, int s01, int s00)
+{
+    const int v = s11 - s10 - s01 + s00;
+    return sizeof(T) == 2 ? (v & 0xFFFF) : v;
+}
+
 // Device words of one score: the maximum's key and the probe (both zero after launch_sat), and
 // the grid bank's template side.
 constexpr int kMaxSlots = 17;

@@ -32,21 +32,6 @@ namespace {
 constexpr int TW = 2;              // warps per block, their tiles side by side in x
 constexpr int NST = 3;             // staged pairs of a warp
 
-__device__ __forceinline__ unsigned long long pack_key(float v, unsigned idx)
-{
-    unsigned b = __float_as_uint(v);
-    b = (b & 0x80000000u) ? ~b : (b | 0x80000000u);   // order-preserving
-    return ((unsigned long long)b << 32) | (unsigned long long)(0xFFFFFFFFu - idx);
-}
-
-// Box count from four integral-image values; exact mod 2^16 for the 16-bit table.
-template <typename T>
-__device__ __forceinline__ int box(int s11, int s10, int s01, int s00)
-{
-    const int v = s11 - s10 - s01 + s00;
-    return sizeof(T) == 2 ? (v & 0xFFFF) : v;
-}
-
 // The integral image, element (y, j, x) at (y * k + j) * P + x, and its coarse samples.
 template <typename T>
 struct Sat {
@@ -148,19 +133,6 @@ __device__ __forceinline__ unsigned long long put_tile(const float (&hs)[TY], in
     return best;
 }
 
-// Asynchronous copies of 16 (past L1) and 4 bytes into shared memory, in commit groups.
-__device__ __forceinline__ void cp16(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp4(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // Grid bank: the shape of a warp's tile and of one staged pair: the four corner blocks of TY rows,
 // each row 32 NX columns from a 16-byte boundary on.
 template <typename T, int NX, int TY>
@@ -258,16 +230,16 @@ __global__ void __launch_bounds__(32 * TW, sizeof(T) == 2 ? 12 : 1) score_grid_t
                 const uint32_t dst = st0 + (uint32_t)ib * L::STAGE;
 #pragma unroll
                 for (int i = 0; i < L::PER; ++i)
-                    if (32 * i + 32 <= L::NCH || lane + 32 * i < L::NCH) cp16(dst + 32 * 16 * i, src + off[i]);
+                    if (32 * i + 32 <= L::NCH || lane + 32 * i < L::NCH) ptx::cp16(dst + 32 * 16 * i, src + off[i]);
             }
-            cp_commit();
+            ptx::cp_commit();
             ib = ib + 1 < NST ? ib + 1 : 0;
         };
 #pragma unroll
         for (int p = 0; p < NST - 1; ++p) issue(p);
         int b = 0;
         for (int p = 0; p < n; ++p) {
-            cp_wait<NST - 2>();
+            ptx::cp_wait<NST - 2>();
             __syncwarp();                                    // every lane's copies have landed, the oldest buffer is read
             issue(p + NST - 1);
             const PairOf<T> e = list[p];
@@ -449,7 +421,7 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
                     from += xq[0];
 #pragma unroll
                     for (int h = 0; h < R; h += 8)
-                        if (c + h < cw) cp16(to + 16 * h, from + h);
+                        if (c + h < cw) ptx::cp16(to + 16 * h, from + h);
                 } else {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -457,13 +429,13 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
                         const int sg = SEP && !outer ? q / 3 : q;
 #pragma unroll
                         for (int h = 0; h < L::CPR; h += 8)
-                            if (c + h < L::CPR) cp16(to + 16 * (sg * L::CPR + h), from + (xq[q] + h));
+                            if (c + h < L::CPR) ptx::cp16(to + 16 * (sg * L::CPR + h), from + (xq[q] + h));
                     }
                 }
             }
-            if (lane < nfg) cp4(dst - 16 * c + lane * 4 + 16 * L::NCH, tcf + j);
+            if (lane < nfg) ptx::cp4(dst - 16 * c + lane * 4 + 16 * L::NCH, tcf + j);
         }
-        cp_commit();
+        ptx::cp_commit();
         ib = ib + 1 < WNST ? ib + 1 : 0;
     };
     float hs[TY];
@@ -500,7 +472,7 @@ __global__ void __launch_bounds__(32 * TW) score_wgrid_tile_kernel(Sat<T> sat, i
         }
 #pragma unroll 1
         for (; p < n && (list[p] >> 8) == g; ++p) {
-            cp_wait<WNST - 2>();
+            ptx::cp_wait<WNST - 2>();
             __syncwarp();
             issue(p + WNST - 1);
             const T *v = reinterpret_cast<const T *>(stage_s[wi][b]);

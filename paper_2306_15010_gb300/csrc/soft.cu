@@ -272,19 +272,6 @@ __global__ void col_box_kernel(const float *__restrict__ RW, int H, int W, int h
     }
 }
 
-// Asynchronous copies of 4 and 16 (past L1) bytes into shared memory, or as many zeros.
-__device__ __forceinline__ void cp4_or_zero(float *dst, const float *src, bool in)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp16_or_zero(float *dst, const float *src, bool in)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // All of a plane's box sums at once: a block takes BXT x BYT outputs, stages the pixels under them,
 // forms the row sums of both widths (the larger is one more, if there are two) from there into
 // shared memory, and from these the column sums of both heights, in the order of row_box_kernel and
@@ -318,10 +305,10 @@ __global__ void __launch_bounds__(256) box_kernel(const float *__restrict__ P, i
     for (int r = warp; r < nr; r += 8) {
         const float *row = src + (size_t)min(y0 + r, H - 1) * W;
         for (int c = lane; c < BXT + wlo; c += 32)
-            cp4_or_zero(ps + r * pc + c, row + min(x0 + c, W - 1), y0 + r < H && x0 + c < W);
+            ptx::cp4_or_zero(ps + r * pc + c, row + min(x0 + c, W - 1), y0 + r < H && x0 + c < W);
     }
-    cp_commit();
-    cp_wait<0>();
+    ptx::cp_commit();
+    ptx::cp_wait<0>();
     __syncthreads();
     for (int e = t; e < nr * (BXT / SEG); e += 256) {
         const int sg = e / nr, r = e - sg * nr;
@@ -697,24 +684,24 @@ __global__ void __launch_bounds__(256) adj_tile_kernel(const float *__restrict__
             const int c = 4 * (t & 15), cx = min(x0 + c, W - 4);
             for (int r = t >> 4; r < nr; r += 16) {
                 const int y = y0 - h + 1 + r;
-                cp16_or_zero(dst + r * BXT + c, src + (size_t)min(max(y, 0), ym) * W + cx, y >= 0 && y <= ym && x0 + c < W);
+                ptx::cp16_or_zero(dst + r * BXT + c, src + (size_t)min(max(y, 0), ym) * W + cx, y >= 0 && y <= ym && x0 + c < W);
             }
         } else {
             for (int r = sg; r < nr; r += 256 / BXT) {
                 const int y = y0 - h + 1 + r;
-                cp4_or_zero(dst + r * BXT + x, src + (size_t)min(max(y, 0), ym) * W + min(gx, W - 1), y >= 0 && y <= ym && gx < W);
+                ptx::cp4_or_zero(dst + r * BXT + x, src + (size_t)min(max(y, 0), ym) * W + min(gx, W - 1), y >= 0 && y <= ym && gx < W);
             }
         }
     };
     stage(0);
-    cp_commit();
+    ptx::cp_commit();
     float out[SEG];
 #pragma unroll
     for (int i = 0; i < SEG; ++i) out[i] = 0.f;
     for (int is = 0; is < ac.ns; ++is) {
         if (is + 1 < ac.ns) stage(is + 1);
-        cp_commit();
-        cp_wait<1>();
+        ptx::cp_commit();
+        ptx::cp_wait<1>();
         __syncthreads();
         const int h = ac.h[is];
         const float *q = bsm + (is & 1) * buf + sg * SEG * BXT + x;
