@@ -91,10 +91,12 @@ typedef struct vqnnf_filter {
     float area;
 } vqnnf_filter;
 
-/* Counters of the near-tie re-scoring, accumulated on the device by vqnnf_assign. */
+/* Counters of one vqnnf_assign call: what its contraction could not decide.  With VQNNF_PREC_FP8 most of
+ * that may be decided by a BF16 pass and only the rest re-scored; the first two still count what the FP8
+ * contraction left. */
 typedef struct vqnnf_assign_stats {
     unsigned long long n_flagged;     /* pixels whose contraction result was ambiguous      */
-    unsigned long long n_candidates;  /* candidate centroids re-scored over those pixels    */
+    unsigned long long n_candidates;  /* candidate centroids of those pixels                */
     unsigned long long n_deep;        /* pixels that needed the double-float second stage   */
     unsigned long long reserved;
 } vqnnf_assign_stats;
@@ -187,7 +189,7 @@ vqnnf_status vqnnf_filter_responses(const uint8_t *labels, int h, int w, int k,
  * for every valid window top-left (y, x), 0 <= y <= H - th, 0 <= x <= W - tw, where
  * q_f(y, x) are the filter's counts over the query NNF with the window at (y, x), taken
  * from the per-cluster integral image of the one-hot query NNF.  The inner sums are exact
- * integers; the outer sum is float32 in bank order.
+ * integers; the outer sum is float32, in bank order (grid banks: in the order of their cells).
  *   q_labels  device, H x W uint8, every label < k;  t_counts: device, F x k int32
  *             (vqnnf_filter_responses)
  *   heatmap   device, (H - th + 1) x (W - tw + 1) float32, written

@@ -151,7 +151,8 @@ def vqnnf_assign(X: torch.Tensor, C: torch.Tensor, prec="fp32", *,
     """H x W uint8 nearest-centroid labels of X (H x W x D float32) over C (k x D).
 
     ``stats``: optional int64 CUDA tensor of 4 words, overwritten with (n_flagged,
-    n_candidates, n_deep, 0) of the near-tie re-scoring.
+    n_candidates, n_deep, 0): the pixels that the contraction left ambiguous, their candidate
+    centroids, and the pixels that needed the double-float stage.
     """
     _need(X, "X", torch.float32)
     _need(C, "C", torch.float32)
